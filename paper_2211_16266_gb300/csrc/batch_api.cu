@@ -39,6 +39,9 @@ struct BatchEngine {
     std::map<TexKey, TexImage> tex;
     std::vector<DevBuffer> ref_stage, out_stage;
     DevBuffer d_problems, d_work, d_counters;
+    DevBuffer d_changed;         // change flags of every keyframe of the batch
+    bool exec_recorded = false;  // a stream being recorded took a replay: its d_changed is kept
+    std::vector<void*> retired;  // outgrown flags that such a recording holds
     void* h_problems = nullptr;  // pinned copies read by the captured graph
     void* h_work = nullptr;
     size_t h_problems_bytes = 0, h_work_bytes = 0;
@@ -101,8 +104,9 @@ void batch_shutdown(pmsp_ctx* c) {
     for (auto* v : {&b.ref_stage, &b.out_stage})
         for (auto& d : *v)
             if (d.ptr) cudaFree(d.ptr);
-    for (DevBuffer* d : {&b.d_problems, &b.d_work, &b.d_counters})
+    for (DevBuffer* d : {&b.d_problems, &b.d_work, &b.d_counters, &b.d_changed})
         if (d->ptr) cudaFree(d->ptr);
+    for (void* p : b.retired) cudaFree(p);
     if (b.h_problems) cudaFreeHost(b.h_problems);
     if (b.h_work) cudaFreeHost(b.h_work);
     if (b.capture) cudaStreamDestroy(b.capture);
@@ -139,6 +143,33 @@ static std::vector<uint8_t> batch_signature(const pmsp_batch_item* items, int n,
         append_bytes(sig, items[i].src_poses, sizeof(pmsp_pose) * items[i].n_src);
     }
     return sig;
+}
+
+// Change flags of the batch's keyframes, n bytes in all, or NULL where there are
+// none (out of memory; a caller's recording, whose replays may overlap a later
+// batch): the half-sweeps then try every neighbour. `own`: the engine's capture,
+// which reuses the flags of the eager run before it.
+static uint8_t* batch_flags(pmsp_ctx* c, BatchEngine& b, size_t n, cudaStream_t st, bool own) {
+    DevBuffer& f = b.d_changed;
+    if (own) return f.bytes >= n ? static_cast<uint8_t*>(f.ptr) : nullptr;
+    if (recording(st)) return nullptr;
+    if (f.bytes < n) {
+        if (f.ptr && b.exec_recorded) {
+            b.retired.push_back(f.ptr);
+            b.exec_recorded = false;
+        } else if (f.ptr) {
+            cudaStreamSynchronize(c->stream);
+            cudaFree(f.ptr);
+        }
+        f = DevBuffer{};
+        if (cudaMalloc(&f.ptr, n) != cudaSuccess) {
+            cudaGetLastError();
+            f.ptr = nullptr;
+            return nullptr;
+        }
+        f.bytes = n;
+    }
+    return static_cast<uint8_t*>(f.ptr);
 }
 
 // Uploads (textures, host references) and the plan; enqueued on `st`.
@@ -206,6 +237,13 @@ static int build_plan(pmsp_ctx* c, BatchEngine& b, const pmsp_batch_item* items,
     }
     c->stream = saved;
     if (rc) return rc;
+    size_t flag_bytes = 0;
+    for (int i = 0; i < n; ++i) flag_bytes += ((size_t)plan.pixels[i] + 255) & ~size_t(255);
+    if (uint8_t* flags = batch_flags(c, b, flag_bytes, st, b.capture && st == b.capture))
+        for (int i = 0; i < n; ++i) {
+            plan.problems[i].changed = flags;
+            flags += ((size_t)plan.pixels[i] + 255) & ~size_t(255);
+        }
 
     // work lists: per phase, the tiles of every keyframe that has that phase
     std::vector<int> ids(n);
@@ -401,6 +439,7 @@ int pmsp_densify_batch(pmsp_ctx* c, const pmsp_batch_item* items, int n, uint32_
             // the replay reads the pinned copies: mark it, unless the caller is recording
             // the stream (an event recorded there could not be waited on afterwards)
             cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
+            b.exec_recorded = b.exec_recorded || recording(c->stream);
             if (e == cudaSuccess && cudaStreamIsCapturing(c->stream, &cap) == cudaSuccess &&
                 cap == cudaStreamCaptureStatusNone) {
                 if (!b.staged_ev) e = cudaEventCreateWithFlags(&b.staged_ev, cudaEventDisableTiming);

@@ -51,6 +51,7 @@ struct alignas(16) PixelParams {
     float* ny;
     float* nz;
     float* cost;
+    uint8_t* changed;     // W*H flags: the pixel's last half-sweep replaced its plane; NULL: no history
     float d_min, d_max;
     float inv_dmin, inv_dmax;
     int S;                // number of sources

@@ -126,6 +126,35 @@ int ensure_buffer(pmsp_ctx* c, DevBuffer& b, size_t bytes) {
     return PMSP_OK;
 }
 
+bool recording(cudaStream_t st) {
+    cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
+    if (cudaStreamIsCapturing(st, &cap) == cudaSuccess) return cap != cudaStreamCaptureStatusNone;
+    cudaGetLastError();
+    return true;
+}
+
+// n bytes of change flags for one densification on the context's stream, or NULL
+// where there are none: out of memory, or a stream being recorded (a replay may
+// run when the context has moved on). The half-sweeps then try every neighbour.
+uint8_t* change_flags(pmsp_ctx* c, size_t n) {
+    DevBuffer& b = c->changed;
+    if (recording(c->stream)) return nullptr;
+    if (b.bytes < n) {
+        if (b.ptr) {
+            cudaStreamSynchronize(c->stream);
+            cudaFree(b.ptr);
+        }
+        b = DevBuffer{};
+        if (cudaMalloc(&b.ptr, n) != cudaSuccess) {
+            cudaGetLastError();
+            b.ptr = nullptr;
+            return nullptr;
+        }
+        b.bytes = n;
+    }
+    return static_cast<uint8_t*>(b.ptr);
+}
+
 void free_texture(TexImage& t) {
     if (t.tex) cudaDestroyTextureObject(t.tex);
     if (t.arr) cudaFreeArray(t.arr);
@@ -414,7 +443,7 @@ int pmsp_destroy(pmsp_ctx* c) {
     runtime_shutdown(c);
     for (auto& t : c->src_tex) free_texture(t);
     free_texture(c->sample_tex);
-    for (DevBuffer* b : {&c->ref_stage, &c->map_stage, &c->filter_stage, &c->sample_stage, &c->median_stage,
+    for (DevBuffer* b : {&c->changed, &c->ref_stage, &c->map_stage, &c->filter_stage, &c->sample_stage, &c->median_stage,
                          &c->warp_zbuf, &c->warp_prev, &c->cloud_table, &c->cloud_stage})
         if (b->ptr) cudaFree(b->ptr);
     if (c->d_err) cudaFree(c->d_err);
@@ -455,6 +484,7 @@ int pmsp_densify(pmsp_ctx* c, const pmsp_image* ref, const pmsp_pose* ref_pose, 
         P.colour = colour;
         if ((rc = launch(c, P, MODE_INIT))) return rc;
     }
+    if (p->iterations > 1) P.changed = change_flags(c, (size_t)P.W * P.H);
     for (int it = 0; it < p->iterations; ++it)
         for (int colour = 0; colour < 2; ++colour) {
             P.colour = colour;
@@ -544,6 +574,7 @@ int pmsp_densify_warped(pmsp_ctx* c, const pmsp_image* ref, const pmsp_pose* ref
     if ((rc = check_maps(c, out, ref->w, ref->h, true, true, "output"))) return rc;
     if ((rc = bind_maps(c, out, P, false))) return rc;
     if ((rc = warp_init_into(c, P, prev, prev_pose, ref_pose, nullptr))) return rc;
+    if (p->iterations > 1) P.changed = change_flags(c, (size_t)P.W * P.H);
     for (int it = 0; it < p->iterations; ++it)
         for (int colour = 0; colour < 2; ++colour) {
             P.colour = colour;

@@ -38,6 +38,8 @@ int check_panorama(pmsp_ctx* c, const pmsp_image* im, const char* what);
 int check_params(pmsp_ctx* c, const pmsp_params* p, int n_src);
 int check_maps(pmsp_ctx* c, const pmsp_maps* m, int W, int H, bool need_normal, bool need_cost, const char* what);
 int ensure_buffer(pmsp_ctx* c, DevBuffer& b, size_t bytes);
+bool recording(cudaStream_t st);  // being captured (or not to be asked about it)
+uint8_t* change_flags(pmsp_ctx* c, size_t n);
 int upload_texture(pmsp_ctx* c, TexImage& t, const pmsp_image* im, cudaStream_t st);
 void free_texture(TexImage& t);
 void compose_rel(const pmsp_pose& r, const pmsp_pose& s, double R[9], double t[3]);
@@ -70,6 +72,7 @@ struct pmsp_ctx {
     pmsp::TexImage sample_tex;
     pmsp::DevBuffer ref_stage, map_stage, filter_stage, sample_stage, median_stage;
     pmsp::DevBuffer cloud_table, cloud_stage;  // fusion (hash table, marks, staging); view filter, completeness
+    pmsp::DevBuffer changed;                   // change flags of the running densification
     pmsp::DevBuffer warp_zbuf, warp_prev;  // plane-map warping: claims, staged previous maps
     pmsp::Serving* serving = nullptr;
     pmsp::BatchEngine* batch = nullptr;

@@ -189,6 +189,7 @@ void fill_request(Serving& s, Request* r) {
     r->prob.ny = base + 2 * N;
     r->prob.nz = base + 3 * N;
     r->prob.cost = base + 4 * N;
+    r->prob.changed = reinterpret_cast<uint8_t*>(base + 5 * N);  // the filtered-depth plane, written only by the tail
     r->prob.err = s.ctx->d_err;
 }
 

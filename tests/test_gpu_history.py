@@ -1,0 +1,102 @@
+"""Whole runs against the same run driven step by step, bit for bit.
+
+Within a run the half-sweeps leave out neighbour candidates that were already
+tried (PixelParams::changed); a half-sweep called on its own has no history and
+tries them all. Both must give the same maps: in one call, warped, batched by
+either strategy, replayed from a graph, and recorded by the caller.
+"""
+import numpy as np
+import pytest
+
+import scenes
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.fixture(scope="module")
+def pm():
+    import __graft_entry__
+    __graft_entry__.build()
+    import paper_2211_16266_gb300 as pm
+    return pm
+
+
+FORMS = [  # W, H, views, format, window, stride, table, best_k, n_refine
+    (96, 48, 1, "u8", 11, 2, 0, 1, 6), (66, 34, 2, "f16", 7, 1, 1, 1, 6), (250, 130, 3, "f32", 9, 3, 1, 2, 6),
+    (8, 4, 2, "u8", 5, 1, 0, 2, 6), (128, 64, 6, "u8", 11, 2, 0, 3, 6), (100, 52, 7, "f32", 11, 2, 1, 7, 0),
+    (64, 34, 10, "f16", 5, 2, 0, 4, 9), (64, 32, 12, "u8", 3, 1, 0, 3, 2), (70, 36, 16, "u8", 21, 5, 0, 16, 1),
+]
+
+
+def _problem(form, n_iter):
+    W, H, S, fmt, pw, st, table, k, nr = form
+    p = scenes.trajectory_problem(W, H, S, seed_scene=1020 + S, fmt=fmt)
+    params = dict(d_min=0.3, d_max=10.0, patch_w=pw, patch_stride=st, iterations=n_iter, best_k=k, sigma_color=0.2,
+                  sigma_space=3.0, n_refine=nr, neighbor_table=table, seed=9, keyframe_id=S)
+    import torch
+    d = lambda a: torch.from_numpy(np.ascontiguousarray(a)).cuda()  # noqa: E731
+    return (d(p.ref.image), (p.ref.R, p.ref.t), [d(f.image) for f in p.srcs], [(f.R, f.t) for f in p.srcs]), params
+
+
+def _steps(pm, ctx, prob, params, start=None):
+    m = start if start is not None else pm.pmsp_init(ctx, *prob, params)
+    for it in range(params["iterations"]):
+        for colour in range(2):
+            pm.pmsp_halfsweep(ctx, *prob, params, colour, it, m)
+    return _bits(pm, ctx, m)
+
+
+def _bits(pm, ctx, m):
+    pm.pmsp_sync(ctx)
+    return [a.cpu().numpy().view(np.uint32).copy() for a in (m.depth, m.normal, m.cost)]
+
+
+def _same(a, b):
+    return all(np.array_equal(x, y) for x, y in zip(a, b))
+
+
+@pytest.mark.parametrize("form", FORMS)
+def test_run_equals_its_steps(pm, form):
+    import torch
+    prob, params = _problem(form, 5)
+    with pm.Context(0) as ctx:
+        want = _steps(pm, ctx, prob, params)
+        for _ in range(2):  # the second run finds the first one's flags
+            assert _same(_bits(pm, ctx, pm.pmsp_densify(ctx, *prob, params)), want)
+        prev = pm.Maps(*[torch.from_numpy(a.view(np.float32)).cuda() for a in want])
+        pose = (np.eye(3), np.array([0.05, 0.0, 0.02]))
+        first = pm.pmsp_warp_init(ctx, *prob, params, prev, pose)
+        warped = _steps(pm, ctx, prob, params, first)
+        assert _same(_bits(pm, ctx, pm.pmsp_densify_warped(ctx, *prob, params, prev, pose)), warped)
+
+
+def test_batches_equal_their_steps(pm):
+    import torch
+    probs = [_problem(FORMS[k], 3 + k % 3) for k in (0, 2, 4, 5, 6)]
+    with pm.Context(0) as ctx:
+        want = [_steps(pm, ctx, *p) for p in probs]
+        for strategy in (0, 1):
+            for flags in (0, pm.PMSP_BATCH_GRAPH):
+                batch = pm.Batch([(*p, params, None) for p, params in probs])
+                t = pm.pmsp_tuning(0, 0, 0, strategy, 0, 1, 0)
+                for _ in range(3):  # eager, captured, replayed
+                    pm.pmsp_densify_batch(ctx, batch, flags, t)
+                for out, w in zip(batch.outs, want):
+                    assert _same(_bits(pm, ctx, out), w)
+    stream = torch.cuda.Stream()
+    with torch.cuda.stream(stream), pm.Context(0, stream=stream) as ctx:  # a run recorded by the caller
+        prob, params = probs[2]
+        out = pm.pmsp_densify(ctx, *prob, params)
+        pm.pmsp_sync(ctx)
+        graph = torch.cuda.CUDAGraph()
+        with torch.cuda.graph(graph, stream=stream):
+            pm.pmsp_densify(ctx, *prob, params, out)
+        # a larger reference against the same sources moves the context's flags (the
+        # recording keeps the source textures, so their sizes stay)
+        big = torch.rand(128, 256, device="cuda")
+        other = pm.pmsp_densify(ctx, big, *prob[1:], params)
+        out.depth.zero_()
+        graph.replay()
+        stream.synchronize()
+        assert _same(_bits(pm, ctx, out), want[2])
+        assert float(other.depth.min()) > 0
