@@ -66,6 +66,7 @@ __global__ void __launch_bounds__(BLOCK_THREADS, min_blocks_for(MAXS)) batch_ker
 template <int MAXS>
 int batch_kernel_blocks_per_sm_t() {
     int n = 0;
+    prefer_texture_cache<batch_kernel<MAXS>>();
     if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, batch_kernel<MAXS>, BLOCK_THREADS, 0) != cudaSuccess)
         return 1;
     return n > 0 ? n : 1;
@@ -74,6 +75,7 @@ int batch_kernel_blocks_per_sm_t() {
 template <int MAXS>
 cudaError_t launch_batch_kernel_t(const BatchArgs& a, int grid, cudaStream_t stream) {
     if (a.n_work <= 0) return cudaSuccess;
+    prefer_texture_cache<batch_kernel<MAXS>>();
     batch_kernel<MAXS><<<grid, BLOCK_THREADS, 0, stream>>>(a);
     return cudaGetLastError();
 }

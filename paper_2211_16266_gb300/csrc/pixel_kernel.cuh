@@ -26,6 +26,8 @@
 
 #include <cuda_fp16.h>
 
+#include <algorithm>
+#include <atomic>
 #include <type_traits>
 
 #include "camera.cuh"
@@ -74,7 +76,7 @@ struct NoPool {};
 // pixels on each side (the window radius the tile serves: the largest, or
 // that of a fixed-window instance); every shape has (TW / 2) x TH pixels of
 // one colour and TPP threads per pixel, 128 threads in all.
-template <int TW, int TH, int TPP = 1, int HALO = MAX_HALO>
+template <int TW, int TH, int TPP = 1, int HALO = MAX_HALO, bool POOL = TPP == 1>
 struct TileSmemT {
     static constexpr int W = TW, H = TH;
     static constexpr int PITCH = TW + 2 * HALO, ROWS = TH + 2 * HALO;
@@ -86,22 +88,22 @@ struct TileSmemT {
     float col_sin[PITCH], col_cos[PITCH];  // sin lon, cos lon
     float wsp[2 * HALO + 1];             // spatial log2-weight of offset index k
     // candidate pooling of the one-thread-per-pixel half-sweep
-    typename std::conditional<TPP == 1, SweepPool, NoPool>::type pool;
+    typename std::conditional<POOL, SweepPool, NoPool>::type pool;
 };
 using TileSmem = TileSmemT<TILE_W, TILE_H>;  // the batched and no-alloc kernels' shape
 
 // Tile shapes of the single-keyframe half-sweep, chosen by PixelParams::tile.
-template <int TS, int HALO = MAX_HALO> struct TileShape { using Smem = TileSmemT<32, 8, 1, HALO>; };
-template <int HALO> struct TileShape<1, HALO> { using Smem = TileSmemT<64, 4, 1, HALO>; };
-template <int HALO> struct TileShape<2, HALO> { using Smem = TileSmemT<16, 16, 1, HALO>; };
+template <int TS, int HALO = MAX_HALO, bool POOL = true> struct TileShape { using Smem = TileSmemT<32, 8, 1, HALO, POOL>; };
+template <int HALO, bool POOL> struct TileShape<1, HALO, POOL> { using Smem = TileSmemT<64, 4, 1, HALO, POOL>; };
+template <int HALO, bool POOL> struct TileShape<2, HALO, POOL> { using Smem = TileSmemT<16, 16, 1, HALO, POOL>; };
 
 // Rotated column directions of the paired path: for view pair q and tile
 // column c, colU[q][k][c] = row k of R_s applied to (sin lon_c, 0, cos lon_c)
 // for both views of the pair. A sample direction r = (cl sin, -sl, cl cos)
-// then transforms as R r = cl U_c - sl R_col1. One table per kernel, sized
-// by the tile's columns (PITCH, halo included) and by CAP pairs: 5 for up to
-// 10 views, so the batched kernel's view counts share one table, and 8 only
-// in the kernels of 11 to 16 views.
+// then transforms as R r = cl U_c - sl R_col1. One table per kernel, sized by the
+// tile's columns (PITCH, halo included) and by the view pairs: the kernels of one
+// view count hold exactly theirs (every KB given up here is texture cache), the
+// batched kernel, whose view counts share one table, five for up to 10 views.
 constexpr int MAX_COL_PAIRS = 5;
 
 template <int CAP, int PITCH>
@@ -110,9 +112,21 @@ __device__ __forceinline__ auto& col_array() {
     return t;
 }
 
-template <int NP, int PITCH>
+struct ParamViews;
+template <int NP, class VA, int PITCH>
 __device__ __forceinline__ auto& col_table() {
-    return col_array<NP <= MAX_COL_PAIRS ? MAX_COL_PAIRS : PMSP_MAX_SOURCES / 2, PITCH>();
+    return col_array<std::is_same<VA, ParamViews>::value ? NP : MAX_COL_PAIRS, PITCH>();
+}
+
+// Loads of read-only shared memory (written before a barrier) at a 32-bit shared
+// address, with the offsets in the instruction. Volatile, so that they are not
+// moved across a barrier.
+__device__ __forceinline__ unsigned shared_at(const void* p) { return (unsigned)__cvta_generic_to_shared(p); }
+template <int OFFSET = 0>
+__device__ __forceinline__ float2 shared_f2(unsigned a) {
+    float2 v;
+    asm volatile("ld.shared.v2.f32 {%0, %1}, [%2+%3];" : "=f"(v.x), "=f"(v.y) : "r"(a), "n"(OFFSET));
+    return v;
 }
 
 // Sample window of the paired cost loop: WIN 0 reads the window from the
@@ -475,17 +489,36 @@ __device__ __forceinline__ float plane_cost(const PixelParams& P, const SM& sm, 
 // gathers are in flight while the next pairs' coordinates are computed; then
 // the interpolation of every pair (2 % faster than pair by pair, and issuing
 // each pair's gathers before the next pair's coordinates another 1.5 %).
-template <int NP, class VA, int PITCH>
+// pairs_columns reads column c's entries of the table from the shared address of
+// its first one; the recursion makes every offset a constant.
+template <int NP, int PITCH, int Q = 0>
+__device__ __forceinline__ void pairs_columns(unsigned col, float2 (&U)[NP][3]) {
+    if constexpr (Q < NP) {
+        U[Q][0] = shared_f2<8 * PITCH * (3 * Q)>(col);
+        U[Q][1] = shared_f2<8 * PITCH * (3 * Q + 1)>(col);
+        U[Q][2] = shared_f2<8 * PITCH * (3 * Q + 2)>(col);
+        pairs_columns<NP, PITCH, Q + 1>(col, U);
+    }
+}
+
+template <int NP, class VA, int PITCH, bool AT_ADDRESS = false>
 __device__ __forceinline__ void pairs_sample(const PixelParams& P, float alpha, float beta, int cx, float2 (&J)[NP]) {
+    float2 U[NP][3];
+    if constexpr (AT_ADDRESS) {
+        pairs_columns<NP, PITCH>(shared_at(&col_table<NP, VA, PITCH>()[0][0][cx]), U);
+    } else {
+#pragma unroll
+        for (int k = 0; k < 3 * NP; ++k) U[k / 3][k % 3] = col_table<NP, VA, PITCH>()[k / 3][k % 3][cx];
+    }
     float2 fx[NP], fy[NP];
     float4 G0[NP], G1[NP];
     const float2 av = pair(alpha), bv = pair(beta);
 #pragma unroll
     for (int q = 0; q < NP; ++q) {
         const auto VP = pair_of<VA>(P.pairs[q]);
-        const float2 Yx = fma2(av, col_table<NP, PITCH>()[q][0][cx], fma2(bv, VP.r1(), VP.t0()));
-        const float2 Yy = fma2(av, col_table<NP, PITCH>()[q][1][cx], fma2(bv, VP.r4(), VP.t1()));
-        const float2 Yz = fma2(av, col_table<NP, PITCH>()[q][2][cx], fma2(bv, VP.r7(), VP.t2()));
+        const float2 Yx = fma2(av, U[q][0], fma2(bv, VP.r1(), VP.t0()));
+        const float2 Yy = fma2(av, U[q][1], fma2(bv, VP.r4(), VP.t1()));
+        const float2 Yz = fma2(av, U[q][2], fma2(bv, VP.r7(), VP.t2()));
         const float2 q2 = fma2(Yx, Yx, mul2(Yz, Yz));
         const float2 rho = make_float2(sqrt_approx(q2.x), sqrt_approx(q2.y));
         const float2 dl = add2(rho, make_float2(fabsf(Yz.x), fabsf(Yz.y)));
@@ -520,7 +553,12 @@ __device__ __forceinline__ void pairs_sample(const PixelParams& P, float alpha, 
 
 // plane_cost for exactly NS >= 2 views held in kernel parameters, with the
 // views processed in pairs (packed FP32) and an odd last view on its own.
-template <int NS, int WIN, class SM, class VA>
+// AT_ADDRESS: the column table by shared addresses, in the half-sweeps of even
+// view counts (1920x960, 6 views, 8 iterations: 76.8 -> 75.8 ms; 3840x1920, 8
+// views: 390 -> 380 ms). With an odd last view, and in the one-evaluation
+// kernels, indexing is the faster (5 views 8.83 against 8.91 ms, the cost of 6
+// views 1.03 against 1.05 ms).
+template <int NS, int WIN, class SM, class VA, bool AT_ADDRESS>
 __device__ __forceinline__ float plane_cost_paired(const PixelParams& P, const SM& sm, int lx, int ly,
                                                    const RefStats& st, float3 rp, float d, float3 n) {
     constexpr int NP = NS / 2;
@@ -542,7 +580,7 @@ __device__ __forceinline__ float plane_cost_paired(const PixelParams& P, const S
         const float t = __fdividef(dn, den);
         const float X = t * rq.x, Y = t * rq.y, Z = t * rq.z;
         const float alpha = t * cl, beta = -t * sm.row_sin[ly + o];
-        pairs_sample<NP, VA, SM::PITCH>(P, alpha, beta, lx + o, c0);
+        pairs_sample<NP, VA, SM::PITCH, AT_ADDRESS>(P, alpha, beta, lx + o, c0);
 #pragma unroll
         for (int q = 0; q < NP; ++q) SJ[q] = SJJ[q] = SIJ[q] = pair(0.f);
         if (ODD) c0o = view_sample<VA>(P.src[NS - 1], X, Y, Z);
@@ -570,7 +608,7 @@ __device__ __forceinline__ float plane_cost_paired(const PixelParams& P, const S
             const float alpha = t * cl, beta = t * msl;
             const float2 w2 = pair(w), wI2 = pair(wI);
             float2 Jall[NP];
-            pairs_sample<NP, VA, SM::PITCH>(P, alpha, beta, cx, Jall);
+            pairs_sample<NP, VA, SM::PITCH, AT_ADDRESS>(P, alpha, beta, cx, Jall);
 #pragma unroll
             for (int q = 0; q < NP; ++q) {
                 const float2 J = Jall[q];
@@ -632,11 +670,11 @@ constexpr bool paired_views() {
 
 // The cost used by the per-pixel kernels: the paired form where the views
 // are exactly known, the general one otherwise.
-template <int NS, bool EXACT, class VA, int WIN = 0, class SM = TileSmem>
+template <int NS, bool EXACT, class VA, int WIN = 0, class SM = TileSmem, bool SWEEP = false>
 __device__ __forceinline__ float cost_of(const PixelParams& P, const SM& sm, int lx, int ly,
                                          const RefStats& st, float3 rp, float d, float3 n) {
     if constexpr (EXACT && NS >= 2 && paired_views<VA>())
-        return plane_cost_paired<NS, WIN, SM, VA>(P, sm, lx, ly, st, rp, d, n);
+        return plane_cost_paired<NS, WIN, SM, VA, SWEEP && NS % 2 == 0>(P, sm, lx, ly, st, rp, d, n);
     else
         return plane_cost<NS, EXACT, VA, SM>(P, sm, lx, ly, st, rp, d, n);
 }
@@ -831,7 +869,7 @@ __device__ __forceinline__ void sweep_pooled(const PixelParams& P, SM& sm, int b
             jrp = make_float3(sm.row_cos[jly] * sm.col_sin[jlx], -sm.row_sin[jly], sm.row_cos[jly] * sm.col_cos[jlx]);
             neighbour_candidate(P, jx, jy, jrp, k, dc, nc);
         }
-        const float c = cost_of<NS, EXACT, VA, WIN, SM>(P, sm, jlx, jly, sm.pool.st[jt], jrp, dc, nc);
+        const float c = cost_of<NS, EXACT, VA, WIN, SM, true>(P, sm, jlx, jly, sm.pool.st[jt], jrp, dc, nc);
         if (r < pooled_rounds) {
             if (c == c) atomicMin(&sm.pool.key[jt], ((unsigned long long)ordered_bits(c) << 3) | (unsigned)k);
         } else if (c < bc) {
@@ -867,9 +905,9 @@ __device__ __forceinline__ void process_tile(const PixelParams& P, SM& sm, int b
             const int q = i / cols, c = i - q * cols;
             const PixelParams::ViewPair& VP = P.pairs[q];
             const float2 sn = pair(sm.col_sin[c]), cs = pair(sm.col_cos[c]);
-            col_table<NP, SM::PITCH>()[q][0][c] = fma2(VP.R[0], sn, mul2(VP.R[2], cs));
-            col_table<NP, SM::PITCH>()[q][1][c] = fma2(VP.R[3], sn, mul2(VP.R[5], cs));
-            col_table<NP, SM::PITCH>()[q][2][c] = fma2(VP.R[6], sn, mul2(VP.R[8], cs));
+            col_table<NP, VA, SM::PITCH>()[q][0][c] = fma2(VP.R[0], sn, mul2(VP.R[2], cs));
+            col_table<NP, VA, SM::PITCH>()[q][1][c] = fma2(VP.R[3], sn, mul2(VP.R[5], cs));
+            col_table<NP, VA, SM::PITCH>()[q][2][c] = fma2(VP.R[6], sn, mul2(VP.R[8], cs));
         }
         __syncthreads();
     }
@@ -906,7 +944,7 @@ __device__ __forceinline__ void process_tile(const PixelParams& P, SM& sm, int b
 
 template <int NS, bool EXACT, int MODE, int WIN = 0, int TS = 0>
 __global__ void __launch_bounds__(BLOCK_THREADS, pixel_min_blocks(NS)) pixel_kernel(const __grid_constant__ PixelParams P) {
-    using SM = typename TileShape<TS, Window<WIN>::HALO>::Smem;
+    using SM = typename TileShape<TS, Window<WIN>::HALO, MODE == MODE_SWEEP>::Smem;
     __shared__ SM sm;
     int tx, ty;
     tile_of_block(gridDim.x, gridDim.y, blockIdx.y * gridDim.x + blockIdx.x, tx, ty);
@@ -920,13 +958,42 @@ inline dim3 tile_grid(const PixelParams& p) {
     return dim3((p.W + SM::W - 1) / SM::W, (p.H + SM::H - 1) / SM::H);
 }
 
+// The split of an SM's 256 KB between shared memory and texture cache that leaves
+// the gathers all but what the blocks that its registers let reside need. The driver's own choice
+// gave shared memory 100 KB where 64 do: 3840x1920 half-sweeps of 8 fp16 views,
+// 4 iterations, took 242.9 ms with 100 KB, 229.0 with 64, 257.1 with 132, 287.0
+// with 164 (1920x960, 6 uint8 views, 8 iterations: 76.4, 76.1, 76.9, 77.7). Set
+// once per kernel and device; a failure leaves the driver's choice.
+template <auto KERNEL>
+inline void prefer_texture_cache() {
+    static std::atomic<uint64_t> done{0};
+    int dev = 0;
+    if (cudaGetDevice(&dev) != cudaSuccess || dev >= 64 || (done.load(std::memory_order_relaxed) >> dev) & 1) return;
+    cudaFuncAttributes a;
+    bool ok = cudaFuncGetAttributes(&a, KERNEL) == cudaSuccess;
+    if (ok) {
+        const int blocks = 65536 / (BLOCK_THREADS * ((a.numRegs + 7) / 8 * 8));
+        const size_t need = (size_t)blocks * (a.sharedSizeBytes + 1024), most = 228 * 1024;  // 1 KB per block is the system's
+        const int percent = (int)std::min<size_t>(100, (100 * need + most - 1) / most);
+        ok = cudaFuncSetAttribute(KERNEL, cudaFuncAttributePreferredSharedMemoryCarveout, percent) == cudaSuccess;
+    }
+    if (!ok) cudaGetLastError();
+    done.fetch_or(1ull << dev, std::memory_order_relaxed);
+}
+
+template <int NS, bool EXACT, int MODE, int WIN = 0, int TS = 0>
+inline void launch_tiles(const PixelParams& p, cudaStream_t stream) {
+    prefer_texture_cache<pixel_kernel<NS, EXACT, MODE, WIN, TS>>();
+    pixel_kernel<NS, EXACT, MODE, WIN, TS><<<tile_grid<TS>(p), BLOCK_THREADS, 0, stream>>>(p);
+}
+
 // A fixed-window sweep in the problem's tile shape.
 template <int NS, bool EXACT, int WIN>
 inline void launch_sweep_window(const PixelParams& p, cudaStream_t stream) {
     switch (p.tile) {
-        case 1: pixel_kernel<NS, EXACT, MODE_SWEEP, WIN, 1><<<tile_grid<1>(p), BLOCK_THREADS, 0, stream>>>(p); break;
-        case 2: pixel_kernel<NS, EXACT, MODE_SWEEP, WIN, 2><<<tile_grid<2>(p), BLOCK_THREADS, 0, stream>>>(p); break;
-        default: pixel_kernel<NS, EXACT, MODE_SWEEP, WIN, 0><<<tile_grid<0>(p), BLOCK_THREADS, 0, stream>>>(p); break;
+        case 1: launch_tiles<NS, EXACT, MODE_SWEEP, WIN, 1>(p, stream); break;
+        case 2: launch_tiles<NS, EXACT, MODE_SWEEP, WIN, 2>(p, stream); break;
+        default: launch_tiles<NS, EXACT, MODE_SWEEP, WIN, 0>(p, stream); break;
     }
 }
 
@@ -947,10 +1014,9 @@ cudaError_t launch_lanes_sweep(const PixelParams& p, cudaStream_t stream);
 
 template <int NS, bool EXACT>
 cudaError_t launch_pixel_kernel_ns(const PixelParams& p, int mode, cudaStream_t stream) {
-    const dim3 grid((p.W + TILE_W - 1) / TILE_W, (p.H + TILE_H - 1) / TILE_H);
     switch (mode) {
-        case MODE_COST: pixel_kernel<NS, EXACT, MODE_COST><<<grid, BLOCK_THREADS, 0, stream>>>(p); break;
-        case MODE_INIT: pixel_kernel<NS, EXACT, MODE_INIT><<<grid, BLOCK_THREADS, 0, stream>>>(p); break;
+        case MODE_COST: launch_tiles<NS, EXACT, MODE_COST>(p, stream); break;
+        case MODE_INIT: launch_tiles<NS, EXACT, MODE_INIT>(p, stream); break;
         default:
             // views split over several warps per pixel (a tuning choice; same maps)
             if constexpr (EXACT && NS >= 2) {
@@ -970,7 +1036,7 @@ cudaError_t launch_pixel_kernel_ns(const PixelParams& p, int mode, cudaStream_t 
                     break;
                 }
             }
-            pixel_kernel<NS, EXACT, MODE_SWEEP><<<grid, BLOCK_THREADS, 0, stream>>>(p);
+            launch_tiles<NS, EXACT, MODE_SWEEP>(p, stream);
             break;
     }
     return cudaGetLastError();

@@ -191,9 +191,9 @@ __global__ void __launch_bounds__(BLOCK_THREADS, pixel_min_blocks(NS))
             const int q = i / cols, c = i - q * cols;
             const PixelParams::ViewPair& VP = P.pairs[q];
             const float2 sn = pair(sm.col_sin[c]), cs = pair(sm.col_cos[c]);
-            col_table<NP, SM::PITCH>()[q][0][c] = fma2(VP.R[0], sn, mul2(VP.R[2], cs));
-            col_table<NP, SM::PITCH>()[q][1][c] = fma2(VP.R[3], sn, mul2(VP.R[5], cs));
-            col_table<NP, SM::PITCH>()[q][2][c] = fma2(VP.R[6], sn, mul2(VP.R[8], cs));
+            col_table<NP, ParamViews, SM::PITCH>()[q][0][c] = fma2(VP.R[0], sn, mul2(VP.R[2], cs));
+            col_table<NP, ParamViews, SM::PITCH>()[q][1][c] = fma2(VP.R[3], sn, mul2(VP.R[5], cs));
+            col_table<NP, ParamViews, SM::PITCH>()[q][2][c] = fma2(VP.R[6], sn, mul2(VP.R[8], cs));
         }
         __syncthreads();
     }
@@ -249,10 +249,13 @@ __global__ void __launch_bounds__(BLOCK_THREADS, pixel_min_blocks(NS))
 template <int NS, int T>
 inline cudaError_t launch_lanes_sweep_t(const PixelParams& p, cudaStream_t stream) {
     const dim3 grid((p.W + 31) / 32, (p.H + 8 / T - 1) / (8 / T));
-    if (window_of(p) == 1)
+    if (window_of(p) == 1) {
+        prefer_texture_cache<pixel_lanes_kernel<NS, T, 1>>();
         pixel_lanes_kernel<NS, T, 1><<<grid, BLOCK_THREADS, 0, stream>>>(p);
-    else
+    } else {
+        prefer_texture_cache<pixel_lanes_kernel<NS, T, 0>>();
         pixel_lanes_kernel<NS, T, 0><<<grid, BLOCK_THREADS, 0, stream>>>(p);
+    }
     return cudaGetLastError();
 }
 

@@ -51,9 +51,9 @@ __device__ __forceinline__ void pairs_sample_sub(const PixelParams& P, float alp
     for (int j = 0; j < NPL; ++j) {
         const int q = SUB + j * T;
         const PixelParams::ViewPair& VP = P.pairs[q];
-        const float2 Yx = fma2(av, col_table<NP, PITCH>()[q][0][cx], fma2(bv, VP.R[1], VP.t[0]));
-        const float2 Yy = fma2(av, col_table<NP, PITCH>()[q][1][cx], fma2(bv, VP.R[4], VP.t[1]));
-        const float2 Yz = fma2(av, col_table<NP, PITCH>()[q][2][cx], fma2(bv, VP.R[7], VP.t[2]));
+        const float2 Yx = fma2(av, col_table<NP, ParamViews, PITCH>()[q][0][cx], fma2(bv, VP.R[1], VP.t[0]));
+        const float2 Yy = fma2(av, col_table<NP, ParamViews, PITCH>()[q][1][cx], fma2(bv, VP.R[4], VP.t[1]));
+        const float2 Yz = fma2(av, col_table<NP, ParamViews, PITCH>()[q][2][cx], fma2(bv, VP.R[7], VP.t[2]));
         const float2 q2 = fma2(Yx, Yx, mul2(Yz, Yz));
         const float2 rho = make_float2(sqrt_approx(q2.x), sqrt_approx(q2.y));
         const float2 dl = add2(rho, make_float2(fabsf(Yz.x), fabsf(Yz.y)));
@@ -250,9 +250,9 @@ __global__ void __launch_bounds__(BLOCK_THREADS, split_min_blocks(NS, T))
             const int q = i / cols, c = i - q * cols;
             const PixelParams::ViewPair& VP = P.pairs[q];
             const float2 sn = pair(sm.col_sin[c]), cs = pair(sm.col_cos[c]);
-            col_table<NP, SM::PITCH>()[q][0][c] = fma2(VP.R[0], sn, mul2(VP.R[2], cs));
-            col_table<NP, SM::PITCH>()[q][1][c] = fma2(VP.R[3], sn, mul2(VP.R[5], cs));
-            col_table<NP, SM::PITCH>()[q][2][c] = fma2(VP.R[6], sn, mul2(VP.R[8], cs));
+            col_table<NP, ParamViews, SM::PITCH>()[q][0][c] = fma2(VP.R[0], sn, mul2(VP.R[2], cs));
+            col_table<NP, ParamViews, SM::PITCH>()[q][1][c] = fma2(VP.R[3], sn, mul2(VP.R[5], cs));
+            col_table<NP, ParamViews, SM::PITCH>()[q][2][c] = fma2(VP.R[6], sn, mul2(VP.R[8], cs));
         }
         __syncthreads();
     }
@@ -333,10 +333,13 @@ __global__ void __launch_bounds__(BLOCK_THREADS, split_min_blocks(NS, T))
 template <int NS, int T>
 inline cudaError_t launch_split_sweep_t(const PixelParams& p, cudaStream_t stream) {
     const dim3 grid((p.W + 31) / 32, (p.H + 8 / T - 1) / (8 / T));
-    if (window_of(p) == 1)
+    if (window_of(p) == 1) {
+        prefer_texture_cache<pixel_split_kernel<NS, T, 1>>();
         pixel_split_kernel<NS, T, 1><<<grid, BLOCK_THREADS, 0, stream>>>(p);
-    else
+    } else {
+        prefer_texture_cache<pixel_split_kernel<NS, T, 0>>();
         pixel_split_kernel<NS, T, 0><<<grid, BLOCK_THREADS, 0, stream>>>(p);
+    }
     return cudaGetLastError();
 }
 
