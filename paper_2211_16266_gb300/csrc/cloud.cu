@@ -8,13 +8,25 @@
 //   atomic add per warp.
 // Fusion: every valid pixel of every keyframe is lifted to a world point and
 //   binned into a cubic voxel; an open-addressing hash table (linear probing,
-//   64-bit packed voxel keys) keeps per voxel the smallest (keyframe, pixel)
-//   order by an atomic minimum. A second pass marks the pixels that are their
-//   voxel's first point, an exclusive scan over the marks gives output slots,
-//   and the marked points are written in (keyframe, pixel) order, so the
-//   output does not depend on thread timing.
+//   64-bit packed voxel keys) keeps per voxel its smallest pixel (numbered through
+//   the keyframes) by an atomic minimum. The kept pixels then set their bit in a
+//   bitmap of all pixels, the bits are counted, and the marked points are written
+//   in (keyframe, pixel) order, so the output does not depend on thread timing.
+//   Bound by the atomics on the table: a wall at 2 m covers a 2 cm voxel with
+//   about 10 pixels of a 1920x960 panorama, so a pixel whose left or upper
+//   neighbour falls into the same voxel (a smaller index: it cannot be the voxel's
+//   first) stays out, and the table is sized for a quarter of the pixels at first
+//   (16 bytes a slot, key and pixel in one sector; 6 keyframes at 1920x960 take
+//   64 MB, within L2, where two slots per pixel took 512 MB). The pixels left are
+//   listed per tile, so that full warps wait for the table together. A table that
+//   fills up is reported and the caller comes again with a larger one. 6 keyframes
+//   at 1920x960, 1 M voxels: 85 us insertion (was 198 over 6 launches), 33 us
+//   marks, scan and points (was 280), against 10 us for its 64 MB of maps, points
+//   and origins; the whole call with its count-only first pass 1.39 -> 0.45 ms.
 // Completeness: one thread per point projects into a W x H panorama and sets
 //   the nearest pixel's flag; a reduction counts the flags.
+#include <algorithm>
+
 #include "camera.cuh"
 #include "common.cuh"
 
@@ -26,8 +38,8 @@ constexpr unsigned long long EMPTY = ~0ull;
 constexpr int KEY_BITS = 21;
 constexpr long long KEY_HALF = 1ll << (KEY_BITS - 1);
 
-__device__ __forceinline__ float3 lift_world(const CloudView& V, int u, int v, float d) {
-    const float3 r = pixel_bearing(u, v, V.W, V.H);
+// World point of range d along the ray r of a pixel.
+__device__ __forceinline__ float3 lift_along(const CloudView& V, float3 r, float d) {
     const float x = fmaf(d, r.x, -V.t[0]), y = fmaf(d, r.y, -V.t[1]), z = fmaf(d, r.z, -V.t[2]);
     // X = R^T (d r - t)
     return make_float3(fmaf(V.R[0], x, fmaf(V.R[3], y, V.R[6] * z)), fmaf(V.R[1], x, fmaf(V.R[4], y, V.R[7] * z)),
@@ -38,11 +50,13 @@ __device__ __forceinline__ float3 lift_world(const CloudView& V, int u, int v, f
 __device__ __forceinline__ bool voxel_key(float3 X, float inv_voxel, unsigned long long& key) {
     const float q[3] = {floorf(X.x * inv_voxel), floorf(X.y * inv_voxel), floorf(X.z * inv_voxel)};
     key = 0;
+    unsigned part[3];
 #pragma unroll
     for (int a = 0; a < 3; ++a) {
         if (!(q[a] >= -(float)KEY_HALF && q[a] < (float)KEY_HALF)) return false;
-        key = (key << KEY_BITS) | (unsigned long long)((long long)q[a] + KEY_HALF);
+        part[a] = (unsigned)((int)q[a] + (int)KEY_HALF);
     }
+    key = ((unsigned long long)part[0] << (2 * KEY_BITS)) | ((unsigned long long)part[1] << KEY_BITS) | part[2];
     return true;
 }
 
@@ -55,134 +69,213 @@ __device__ __forceinline__ unsigned long long hash_slot(unsigned long long key, 
     return key & mask;
 }
 
-__global__ void fuse_insert_kernel(const __grid_constant__ FuseArgs A, int k) {
-    const CloudView& V = A.views[k];
-    const int i = blockIdx.x * blockDim.x + threadIdx.x;
-    if (i >= V.W * V.H) return;
-    const float d = V.depth[i];
-    if (!(d > 0.f)) return;
-    const float3 X = lift_world(V, i % V.W, i / V.W, d);
-    unsigned long long key;
-    if (!voxel_key(X, A.inv_voxel, key)) {
-        atomicOr(A.err, ERR_RANGE);
-        return;
-    }
-    const unsigned long long order = ((unsigned long long)k << 32) | (unsigned)i;
-    unsigned long long s = hash_slot(key, A.mask);
-    for (unsigned long long probe = 0; probe <= A.mask; ++probe) {  // bounded: at most one pass over the table
-        const unsigned long long prev = atomicCAS(A.keys + s, EMPTY, key);
-        if (prev == EMPTY || prev == key) {
-            atomicMin(A.vals + s, order);
-            return;
-        }
-        s = (s + 1) & A.mask;
-    }
-    atomicOr(A.err, ERR_CAPACITY);
+constexpr int FT_W = 32, FT_H = 8, FT_V = 4;  // threads of a block, pixels of a thread (every eighth row of a 32 x 32 tile)
+// Keyframe and tile of block b: the keyframes' tiles are numbered one after another.
+__device__ __forceinline__ int fuse_view(const FuseArgs& A, int b) {
+    int k = 0;
+    while (k + 1 < A.n && b >= A.tile_base[k + 1]) ++k;
+    return k;
 }
 
-__global__ void fuse_mark_kernel(const __grid_constant__ FuseArgs A, int k, unsigned* mark) {
+__global__ void __launch_bounds__(FT_W * FT_H) fuse_insert_kernel(const __grid_constant__ FuseArgs A) {
+    __shared__ float2 row[FT_H * FT_V], col[FT_W];  // (sin, cos) of latitude and longitude, as pixel_bearing
+    __shared__ unsigned long long keys[FT_H * FT_V][FT_W];
+    __shared__ unsigned short list[FT_H * FT_V * FT_W];
+    __shared__ unsigned claimed, full, listed;
+    const int k = fuse_view(A, blockIdx.x), b = blockIdx.x - A.tile_base[k];
     const CloudView& V = A.views[k];
-    const int i = blockIdx.x * blockDim.x + threadIdx.x;
-    if (i >= V.W * V.H) return;
-    unsigned m = 0;
-    const float d = V.depth[i];
-    if (d > 0.f) {
-        const float3 X = lift_world(V, i % V.W, i / V.W, d);
-        unsigned long long key;
-        if (voxel_key(X, A.inv_voxel, key)) {
-            const unsigned long long order = ((unsigned long long)k << 32) | (unsigned)i;
-            unsigned long long s = hash_slot(key, A.mask);
-            for (unsigned long long probe = 0; probe <= A.mask; ++probe) {
-                const unsigned long long kk = A.keys[s];
-                if (kk == key) {
-                    m = A.vals[s] == order;
-                    break;
-                }
-                if (kk == EMPTY) break;
-                s = (s + 1) & A.mask;
+    const int tiles_x = (V.W + FT_W - 1) / FT_W;
+    const int u0 = (b % tiles_x) * FT_W, v0 = (b / tiles_x) * FT_H * FT_V;
+    const int u = u0 + threadIdx.x, tid = threadIdx.y * FT_W + threadIdx.x;
+    float d[FT_V];
+#pragma unroll
+    for (int p = 0; p < FT_V; ++p) {
+        const int v = v0 + threadIdx.y + p * FT_H;
+        d[p] = u < V.W && v < V.H ? V.depth[v * V.W + u] : 0.f;
+    }
+    if (tid < FT_W + FT_H * FT_V) {
+        float sn, cs;
+        if (tid < FT_W) {
+            sincospif((2.0f * (u0 + tid) + 1.0f) / V.W - 1.0f, &sn, &cs);
+            col[tid] = make_float2(sn, cs);
+        } else {
+            sincospif(0.5f - (2.0f * (v0 + tid - FT_W) + 1.0f) / (2.0f * V.H), &sn, &cs);
+            row[tid - FT_W] = make_float2(sn, cs);
+        }
+    } else if (tid == FT_W * FT_H - 1) {
+        claimed = listed = 0;
+        full = *(volatile unsigned*)A.err & ERR_CAPACITY;  // the caller will come again: nothing more is worth doing
+        if (!full && *(volatile unsigned long long*)A.count > A.most_voxels) {
+            full = 1;
+            atomicOr(A.err, ERR_CAPACITY);
+        }
+    }
+    __syncthreads();
+    unsigned long long key[FT_V];
+#pragma unroll
+    for (int p = 0; p < FT_V; ++p) {
+        key[p] = EMPTY;
+        if (d[p] > 0.f) {
+            const float2 r = row[threadIdx.y + p * FT_H], c = col[threadIdx.x];
+            const float3 X = lift_along(V, make_float3(r.y * c.x, -r.x, r.y * c.y), d[p]);
+            if (!voxel_key(X, A.inv_voxel, key[p])) {
+                key[p] = EMPTY;
+                atomicOr(A.err, ERR_RANGE);
             }
         }
+        keys[threadIdx.y + p * FT_H][threadIdx.x] = key[p];
     }
-    mark[A.base[k] + i] = m;
+    __syncthreads();
+    if (full) return;
+    // the tile's candidates in a list, so that the insertion runs with full warps
+#pragma unroll
+    for (int p = 0; p < FT_V; ++p) {
+        const int y = threadIdx.y + p * FT_H;
+        bool first = key[p] != EMPTY;
+        if (first && threadIdx.x > 0) first = keys[y][threadIdx.x - 1] != key[p];
+        if (first && y > 0) first = keys[y - 1][threadIdx.x] != key[p];
+        const unsigned m = __ballot_sync(0xffffffffu, first);
+        unsigned at = 0;
+        if (threadIdx.x == 0 && m) at = atomicAdd(&listed, __popc(m));
+        at = __shfl_sync(0xffffffffu, at, 0) + __popc(m & ((1u << threadIdx.x) - 1u));
+        if (first) list[at] = (unsigned short)(y * FT_W + threadIdx.x);
+    }
+    __syncthreads();
+    unsigned won = 0;
+    for (int c = tid; c < (int)listed; c += FT_W * FT_H) {
+        const int y = list[c] / FT_W, x = list[c] % FT_W;
+        const unsigned long long mine = keys[y][x];
+        unsigned long long s = hash_slot(mine, A.mask), probe = 0;
+        for (; probe < A.most_probes; ++probe) {  // bounded: at most one pass over the table
+            FuseSlot* t = A.table + s;
+            unsigned long long seen = *(volatile unsigned long long*)&t->key;
+            if (seen == EMPTY) {
+                seen = atomicCAS(&t->key, EMPTY, mine);
+                won += seen == EMPTY;
+            }
+            if (seen == EMPTY || seen == mine) {
+                atomicMin(&t->pixel, (unsigned)(A.base[k] + (v0 + y) * V.W + u0 + x));
+                break;
+            }
+            s = (s + 1) & A.mask;
+        }
+        if (probe == A.most_probes) atomicOr(A.err, ERR_CAPACITY);
+    }
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) won += __shfl_xor_sync(0xffffffffu, won, o);
+    if (threadIdx.x == 0 && won) atomicAdd(&claimed, won);
+    __syncthreads();
+    if (tid == 0 && claimed) atomicAdd(A.count, (unsigned long long)claimed);
 }
 
-// Exclusive scan of n marks in three passes: per-block sums, a single-block
-// scan of the block sums, then per-block scans offset by their block's sum.
-constexpr int SCAN_BLOCK = 1024;
+// Sets the bit of every slot's pixel.
+__global__ void __launch_bounds__(256) fuse_mark_kernel(const __grid_constant__ FuseArgs A) {
+    for (unsigned long long s = (unsigned long long)blockIdx.x * 256 + threadIdx.x; s <= A.mask; s += (unsigned long long)gridDim.x * 256) {
+        const ulonglong2 t = *reinterpret_cast<const ulonglong2*>(A.table + s);
+        if (t.x == EMPTY) continue;
+        const unsigned p = (unsigned)t.y;
+        atomicOr(A.bits + (p >> 5), 1u << (p & 31));
+    }
+}
 
-__device__ __forceinline__ unsigned block_exclusive_scan(unsigned x, unsigned* warp_sums, unsigned& total) {
-    const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
-    unsigned incl = x;
+constexpr int SCAN_BLOCK = 256;  // bitmap words (32 pixels each) of a block of the two passes below
+
+__device__ __forceinline__ unsigned block_sum(unsigned x, unsigned* warp_sums) {
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) x += __shfl_xor_sync(0xffffffffu, x, o);
+    if ((threadIdx.x & 31) == 0) warp_sums[threadIdx.x >> 5] = x;
+    __syncthreads();
+    unsigned s = 0;
+    for (int w = 0; w < SCAN_BLOCK / 32; ++w) s += warp_sums[w];
+    __syncthreads();
+    return s;
+}
+
+__global__ void __launch_bounds__(SCAN_BLOCK) fuse_count_kernel(const __grid_constant__ FuseArgs A) {
+    __shared__ unsigned ws[SCAN_BLOCK / 32];
+    const int w = blockIdx.x * SCAN_BLOCK + threadIdx.x;
+    const unsigned s = block_sum(w < A.n_words ? __popc(A.bits[w]) : 0, ws);
+    if (threadIdx.x == 0) A.sums[blockIdx.x] = s;
+}
+
+// The groups' sums to the marks before each group, by one block.
+__global__ void __launch_bounds__(1024) fuse_scan_kernel(unsigned* sums, int groups) {
+    __shared__ unsigned ws[32];
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    unsigned carry = 0;
+    for (int c = 0; c < groups; c += 1024) {
+        const int q = c + threadIdx.x;
+        const unsigned x = q < groups ? sums[q] : 0;
+        unsigned incl = x;
+#pragma unroll
+        for (int o = 1; o < 32; o <<= 1) {
+            const unsigned y = __shfl_up_sync(0xffffffffu, incl, o);
+            if (lane >= o) incl += y;
+        }
+        if (lane == 31) ws[warp] = incl;
+        __syncthreads();
+        unsigned before = carry;
+        for (int w = 0; w < warp; ++w) before += ws[w];
+        if (q < groups) sums[q] = before + incl - x;
+        for (int w = 0; w < 32; ++w) carry += ws[w];
+        __syncthreads();
+    }
+}
+
+// Writes the marked points of a group of 256 words, a thread per point: its word
+// by bisection of the marks before each, its bit within the word by halving.
+// (A lane per pixel instead kept 3 of 32 lanes busy: 53 us for what takes 12.)
+__global__ void __launch_bounds__(SCAN_BLOCK) fuse_write_kernel(const __grid_constant__ FuseArgs A) {
+    __shared__ unsigned ws[SCAN_BLOCK / 32], words[SCAN_BLOCK], before[SCAN_BLOCK];
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    const int w0 = blockIdx.x * SCAN_BLOCK;
+    const unsigned own = w0 + threadIdx.x < A.n_words ? A.bits[w0 + threadIdx.x] : 0;
+    unsigned incl = __popc(own);
+    const unsigned mine = incl;
 #pragma unroll
     for (int o = 1; o < 32; o <<= 1) {
         const unsigned y = __shfl_up_sync(0xffffffffu, incl, o);
         if (lane >= o) incl += y;
     }
-    if (lane == 31) warp_sums[w] = incl;
+    if (lane == 31) ws[warp] = incl;
     __syncthreads();
-    if (w == 0) {
-        unsigned s = lane < (int)(blockDim.x >> 5) ? warp_sums[lane] : 0;
+    unsigned ahead = 0, total = 0;
+    for (int w = 0; w < SCAN_BLOCK / 32; ++w) {
+        if (w < warp) ahead += ws[w];
+        total += ws[w];
+    }
+    words[threadIdx.x] = own;
+    before[threadIdx.x] = ahead + incl - mine;
+    __syncthreads();
+    const long long start = A.sums[blockIdx.x];
+    for (unsigned q = threadIdx.x; q < total && start + q < A.cap; q += SCAN_BLOCK) {
+        int w = 0;
 #pragma unroll
-        for (int o = 1; o < 32; o <<= 1) {
-            const unsigned y = __shfl_up_sync(0xffffffffu, s, o);
-            if (lane >= o) s += y;
+        for (int h = SCAN_BLOCK / 2; h > 0; h >>= 1)
+            if (before[w + h] <= q) w += h;  // the last word with at most q marks before it has the mark
+        unsigned bits = words[w], n = q - before[w];
+        int bit = 0;
+#pragma unroll
+        for (int h = 16; h > 0; h >>= 1) {
+            const unsigned c = __popc(bits & ((1u << h) - 1u));
+            if (n >= c) {
+                n -= c;
+                bits >>= h;
+                bit += h;
+            }
         }
-        warp_sums[lane] = s;  // inclusive prefix of warp sums
+        const long long g = ((long long)(w0 + w) << 5) + bit;  // pixel, numbered through the keyframes
+        int k = 0;
+        while (k + 1 < A.n && g >= A.base[k + 1]) ++k;
+        const CloudView& V = A.views[k];
+        const int i = (int)(g - A.base[k]);
+        const float3 X = lift_along(V, pixel_bearing(i % V.W, i / V.W, V.W, V.H), V.depth[i]);
+        float* o = A.points + 3 * (start + q);
+        o[0] = X.x;
+        o[1] = X.y;
+        o[2] = X.z;
+        if (A.src) A.src[start + q] = (long long)(((unsigned long long)k << 32) | (unsigned)i);
     }
-    __syncthreads();
-    total = warp_sums[(blockDim.x >> 5) - 1];
-    const unsigned before = w > 0 ? warp_sums[w - 1] : 0;
-    return before + incl - x;
-}
-
-__global__ void __launch_bounds__(SCAN_BLOCK) scan_block_sums(const unsigned* mark, long long n, unsigned* sums) {
-    __shared__ unsigned ws[32];
-    const long long i = (long long)blockIdx.x * SCAN_BLOCK + threadIdx.x;
-    const unsigned x = i < n ? mark[i] : 0;
-    unsigned total;
-    block_exclusive_scan(x, ws, total);
-    if (threadIdx.x == 0) sums[blockIdx.x] = total;
-}
-
-// One block: exclusive scan of nb block sums in place (chunks of SCAN_BLOCK);
-// total written to *count.
-__global__ void __launch_bounds__(SCAN_BLOCK) scan_sums(unsigned* sums, int nb, unsigned long long* count) {
-    __shared__ unsigned ws[32];
-    unsigned carry = 0;
-    for (int c = 0; c < nb; c += SCAN_BLOCK) {
-        const int i = c + threadIdx.x;
-        const unsigned x = i < nb ? sums[i] : 0;
-        unsigned total;
-        const unsigned ex = block_exclusive_scan(x, ws, total);
-        if (i < nb) sums[i] = carry + ex;
-        carry += total;
-        __syncthreads();
-    }
-    if (threadIdx.x == 0) *count = carry;
-}
-
-__global__ void __launch_bounds__(SCAN_BLOCK) scan_apply(unsigned* mark, long long n, const unsigned* sums) {
-    __shared__ unsigned ws[32];
-    const long long i = (long long)blockIdx.x * SCAN_BLOCK + threadIdx.x;
-    const unsigned x = i < n ? mark[i] : 0;
-    unsigned total;
-    const unsigned ex = block_exclusive_scan(x, ws, total);
-    // marks become output positions + 1 (0: not kept)
-    if (i < n) mark[i] = x ? sums[blockIdx.x] + ex + 1 : 0;
-}
-
-__global__ void fuse_write_kernel(const __grid_constant__ FuseArgs A, int k, const unsigned* pos) {
-    const CloudView& V = A.views[k];
-    const int i = blockIdx.x * blockDim.x + threadIdx.x;
-    if (i >= V.W * V.H) return;
-    const unsigned p = pos[A.base[k] + i];
-    if (p == 0 || (long long)(p - 1) >= A.cap) return;
-    const float3 X = lift_world(V, i % V.W, i / V.W, V.depth[i]);
-    float* o = A.points + 3 * (size_t)(p - 1);
-    o[0] = X.x;
-    o[1] = X.y;
-    o[2] = X.z;
-    if (A.src) A.src[p - 1] = (long long)(((unsigned long long)k << 32) | (unsigned)i);
 }
 
 __global__ void completeness_kernel(const __grid_constant__ CompletenessArgs A) {
@@ -232,26 +325,21 @@ __global__ void view_filter_kernel(const __grid_constant__ ViewFilterArgs A) {
 
 }  // namespace
 
-cudaError_t launch_fuse(const FuseArgs& a, int n, unsigned* mark, unsigned* sums, long long total,
-                        unsigned long long* count, cudaStream_t stream) {
-    cudaError_t e = cudaMemsetAsync(a.keys, 0xff, (a.mask + 1) * sizeof(unsigned long long), stream);
-    if (e == cudaSuccess) e = cudaMemsetAsync(a.vals, 0xff, (a.mask + 1) * sizeof(unsigned long long), stream);
+int fuse_tiles(int W, int H) { return ((W + FT_W - 1) / FT_W) * ((H + FT_H * FT_V - 1) / (FT_H * FT_V)); }
+
+cudaError_t launch_fuse(const FuseArgs& a, cudaStream_t stream) {
+    cudaError_t e = cudaMemsetAsync(a.table, 0xff, (a.mask + 1) * sizeof(FuseSlot), stream);
+    if (e == cudaSuccess) e = cudaMemsetAsync(a.count, 0, 2 * sizeof(unsigned long long), stream);  // and the error word
     if (e != cudaSuccess) return e;
-    for (int k = 0; k < n; ++k) {
-        const int px = a.views[k].W * a.views[k].H;
-        fuse_insert_kernel<<<(px + 255) / 256, 256, 0, stream>>>(a, k);
-    }
-    for (int k = 0; k < n; ++k) {
-        const int px = a.views[k].W * a.views[k].H;
-        fuse_mark_kernel<<<(px + 255) / 256, 256, 0, stream>>>(a, k, mark);
-    }
-    const int nb = (int)((total + SCAN_BLOCK - 1) / SCAN_BLOCK);
-    scan_block_sums<<<nb, SCAN_BLOCK, 0, stream>>>(mark, total, sums);
-    scan_sums<<<1, SCAN_BLOCK, 0, stream>>>(sums, nb, count);
-    scan_apply<<<nb, SCAN_BLOCK, 0, stream>>>(mark, total, sums);
-    for (int k = 0; k < n; ++k) {
-        const int px = a.views[k].W * a.views[k].H;
-        fuse_write_kernel<<<(px + 255) / 256, 256, 0, stream>>>(a, k, mark);
+    fuse_insert_kernel<<<a.tile_base[a.n], dim3(FT_W, FT_H), 0, stream>>>(a);
+    if (a.cap > 0) {  // else the count is all that is asked for
+        e = cudaMemsetAsync(a.bits, 0, (size_t)a.n_words * sizeof(unsigned), stream);
+        if (e != cudaSuccess) return e;
+        const int blocks = (a.n_words + SCAN_BLOCK - 1) / SCAN_BLOCK;
+        fuse_mark_kernel<<<(unsigned)std::min<unsigned long long>((a.mask + 256) / 256, 8192), 256, 0, stream>>>(a);
+        fuse_count_kernel<<<blocks, SCAN_BLOCK, 0, stream>>>(a);
+        fuse_scan_kernel<<<1, 1024, 0, stream>>>(a.sums, blocks);
+        fuse_write_kernel<<<blocks, SCAN_BLOCK, 0, stream>>>(a);
     }
     return cudaGetLastError();
 }

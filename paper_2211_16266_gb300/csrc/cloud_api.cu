@@ -2,6 +2,7 @@
 // fusion and keyframe completeness. Host buffers are staged through context
 // buffers; every call returns after its results are on the host side of the
 // caller (counts are always read back).
+#include <algorithm>
 #include <cmath>
 #include <cstring>
 
@@ -100,68 +101,83 @@ int pmsp_fuse(pmsp_ctx* c, const pmsp_maps* maps, const pmsp_pose* poses, int n,
         total += (long long)maps[k].w * maps[k].h;
     }
     if (total >= (1ll << 31)) return ctx_fail(c, PMSP_EINVAL, "too many pixels to fuse in one call");
-    unsigned long long slots = 1024;
-    while (slots < 2ull * (unsigned long long)total) slots <<= 1;
-    const int nb = (int)((total + 1023) / 1024);
+    // The table starts at a slot for every fourth pixel (dense maps put several
+    // pixels into a voxel) and grows fourfold, to at most two slots per pixel, as
+    // long as the insertion reports it too small.
+    unsigned long long slots = 1024, most = 1024;
+    while (most < 2ull * (unsigned long long)total) most <<= 1;
+    while (slots < (unsigned long long)total / 4) slots <<= 1;
     const bool host = memory == PMSP_HOST;
     const long long kept_max = cap < total ? cap : total;
-    // context buffers: hash table | marks | block sums | count + error | host staging
-    const size_t t_bytes = rounded(2 * slots * sizeof(unsigned long long));
-    const size_t m_bytes = rounded((size_t)total * sizeof(unsigned)), s_bytes = rounded((size_t)nb * sizeof(unsigned));
-    const size_t c_bytes = rounded(2 * sizeof(unsigned long long));
-    size_t h_bytes = 0;
-    if (host)
-        h_bytes = rounded((size_t)total * sizeof(float)) + rounded((size_t)kept_max * 3 * sizeof(float)) +
-                  rounded((size_t)kept_max * sizeof(long long));
-    int rc;
-    if ((rc = ensure_buffer(c, c->cloud_table, t_bytes + m_bytes + s_bytes + c_bytes + h_bytes))) return rc;
-    char* base = static_cast<char*>(c->cloud_table.ptr);
+    const int n_words = (int)((total + 31) / 32);
     FuseArgs A;
     memset(&A, 0, sizeof A);
-    A.keys = reinterpret_cast<unsigned long long*>(base);
-    A.vals = A.keys + slots;
-    A.mask = slots - 1;
-    unsigned* mark = reinterpret_cast<unsigned*>(base + t_bytes);
-    unsigned* sums = reinterpret_cast<unsigned*>(base + t_bytes + m_bytes);
-    unsigned long long* d_count = reinterpret_cast<unsigned long long*>(base + t_bytes + m_bytes + s_bytes);
-    A.err = reinterpret_cast<unsigned*>(d_count + 1);
-    char* hs = base + t_bytes + m_bytes + s_bytes + c_bytes;
-    A.inv_voxel = 1.0f / voxel;
-    A.cap = cap;
-    A.points = points;
-    A.src = reinterpret_cast<long long*>(src);
-    if (host) {
-        A.points = reinterpret_cast<float*>(hs + rounded((size_t)total * sizeof(float)));
-        A.src = src ? reinterpret_cast<long long*>(hs + rounded((size_t)total * sizeof(float)) +
-                                                   rounded((size_t)kept_max * 3 * sizeof(float)))
-                    : nullptr;
-        A.cap = kept_max;
-    }
-    cudaError_t e = cudaMemsetAsync(A.err, 0, sizeof(unsigned), c->stream);
-    if (e != cudaSuccess) return cuda_fail(c, e, "fuse setup");
-    long long off = 0;
-    for (int k = 0; k < n; ++k) {
-        CloudView& V = A.views[k];
-        V.W = maps[k].w;
-        V.H = maps[k].h;
-        V.depth = maps[k].depth;
-        const size_t px = (size_t)V.W * V.H;
-        if (host) {
-            float* d = reinterpret_cast<float*>(hs) + off;
-            if ((rc = stage_in(c, maps[k].depth, px, d))) return rc;
-            V.depth = d;
-        }
-        for (int j = 0; j < 9; ++j) V.R[j] = (float)poses[k].R[j];
-        for (int j = 0; j < 3; ++j) V.t[j] = (float)poses[k].t[j];
-        A.base[k] = off;
-        off += (long long)px;
-    }
-    e = launch_fuse(A, n, mark, sums, total, d_count, c->stream);
-    if (e != cudaSuccess) return cuda_fail(c, e, "fuse launch");
     unsigned long long res[2] = {0, 0};
-    e = cudaMemcpyAsync(res, d_count, sizeof res, cudaMemcpyDeviceToHost, c->stream);
-    if (e == cudaSuccess) e = cudaStreamSynchronize(c->stream);
-    if (e != cudaSuccess) return cuda_fail(c, e, "fuse read-back");
+    int rc;
+    for (;;) {
+        // context buffers: hash table | bits | block sums | count + error | host staging
+        const size_t t_bytes = rounded(slots * sizeof(FuseSlot)), b_bytes = rounded((size_t)n_words * sizeof(unsigned));
+        const size_t s_bytes = rounded(((size_t)n_words / 256 + 1) * sizeof(unsigned));
+        const size_t c_bytes = rounded(2 * sizeof(unsigned long long));
+        size_t h_bytes = 0;
+        if (host)
+            h_bytes = rounded((size_t)total * sizeof(float)) + rounded((size_t)kept_max * 3 * sizeof(float)) +
+                      rounded((size_t)kept_max * sizeof(long long));
+        if ((rc = ensure_buffer(c, c->cloud_table, t_bytes + b_bytes + s_bytes + c_bytes + h_bytes))) return rc;
+        char* base = static_cast<char*>(c->cloud_table.ptr);
+        A.table = reinterpret_cast<FuseSlot*>(base);
+        A.mask = slots - 1;
+        A.most_probes = slots < most ? 128 : slots;
+        A.most_voxels = slots < most ? slots - slots / 4 : slots;
+        A.bits = reinterpret_cast<unsigned*>(base + t_bytes);
+        A.n_words = n_words;
+        A.sums = reinterpret_cast<unsigned*>(base + t_bytes + b_bytes);
+        A.count = reinterpret_cast<unsigned long long*>(base + t_bytes + b_bytes + s_bytes);
+        A.err = reinterpret_cast<unsigned*>(A.count + 1);
+        char* hs = base + t_bytes + b_bytes + s_bytes + c_bytes;
+        A.inv_voxel = 1.0f / voxel;
+        A.cap = cap;
+        A.points = points;
+        A.src = reinterpret_cast<long long*>(src);
+        if (host) {
+            A.points = reinterpret_cast<float*>(hs + rounded((size_t)total * sizeof(float)));
+            A.src = src ? reinterpret_cast<long long*>(hs + rounded((size_t)total * sizeof(float)) +
+                                                       rounded((size_t)kept_max * 3 * sizeof(float)))
+                        : nullptr;
+            A.cap = kept_max;
+        }
+        A.n = n;
+        long long off = 0;
+        int tiles = 0;
+        for (int k = 0; k < n; ++k) {
+            CloudView& V = A.views[k];
+            V.W = maps[k].w;
+            V.H = maps[k].h;
+            V.depth = maps[k].depth;
+            const size_t px = (size_t)V.W * V.H;
+            if (host) {  // (a larger buffer moved the staging)
+                float* d = reinterpret_cast<float*>(hs) + off;
+                if ((rc = stage_in(c, maps[k].depth, px, d))) return rc;
+                V.depth = d;
+            }
+            for (int j = 0; j < 9; ++j) V.R[j] = (float)poses[k].R[j];
+            for (int j = 0; j < 3; ++j) V.t[j] = (float)poses[k].t[j];
+            A.base[k] = off;
+            A.tile_base[k] = tiles;
+            off += (long long)px;
+            tiles += fuse_tiles(V.W, V.H);
+        }
+        A.base[n] = off;
+        A.tile_base[n] = tiles;
+        cudaError_t e = launch_fuse(A, c->stream);
+        if (e != cudaSuccess) return cuda_fail(c, e, "fuse launch");
+        e = cudaMemcpyAsync(res, A.count, sizeof res, cudaMemcpyDeviceToHost, c->stream);
+        if (e == cudaSuccess) e = cudaStreamSynchronize(c->stream);
+        if (e != cudaSuccess) return cuda_fail(c, e, "fuse read-back");
+        if (((unsigned)res[1] & ERR_RANGE) || !((unsigned)res[1] & ERR_CAPACITY) || slots >= most) break;
+        slots = std::min(most, slots * 4);
+    }
+    cudaError_t e = cudaSuccess;
     const unsigned err = (unsigned)res[1];
     if (err & ERR_RANGE) return ctx_fail(c, PMSP_EINVAL, "a point lies more than 2^20 voxels from the origin");
     if (err) return ctx_fail(c, PMSP_EDEVICE, "fuse error flag 0x%x", err);

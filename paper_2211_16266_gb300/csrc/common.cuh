@@ -120,16 +120,28 @@ struct CloudView {
 
 constexpr int MAX_FUSE_VIEWS = PMSP_MAX_SOURCES;
 
+struct alignas(16) FuseSlot {
+    unsigned long long key;  // packed voxel key, ~0 = empty
+    unsigned pixel;          // smallest pixel of the voxel, numbered through the keyframes
+    unsigned pad;
+};
+
 struct FuseArgs {
     CloudView views[MAX_FUSE_VIEWS];
-    long long base[MAX_FUSE_VIEWS];  // offset of each keyframe's pixels in the mark array
+    long long base[MAX_FUSE_VIEWS + 1];  // number of each keyframe's first pixel
+    int tile_base[MAX_FUSE_VIEWS + 1];   // and tile
+    int n;
     float inv_voxel;
-    unsigned long long* keys;        // hash table: packed voxel keys, ~0 = empty
-    unsigned long long* vals;        // smallest (keyframe << 32 | pixel) per voxel
+    FuseSlot* table;
     unsigned long long mask;         // table capacity - 1 (capacity a power of two)
+    unsigned long long most_probes, most_voxels;  // beyond either the table counts as too small
+    unsigned* bits;                  // a bit per pixel: kept
+    int n_words;
+    unsigned* sums;                  // kept pixels per group of 256 words, then before it
     float* points;                   // output: 3 floats per kept point
     long long* src;                  // output (optional): keyframe << 32 | pixel
     long long cap;                   // output capacity in points
+    unsigned long long* count;       // voxels; the error word follows it
     unsigned* err;
 };
 
@@ -171,8 +183,8 @@ cudaError_t launch_filter_kernel(const FilterParams& p, cudaStream_t stream);
 cudaError_t launch_median_kernel(const float* in, float* out, int W, int H, int radius, float tau,
                                  cudaStream_t stream);
 cudaError_t launch_warp_init(const PixelParams& p, const WarpArgs& a, cudaStream_t stream);
-cudaError_t launch_fuse(const FuseArgs& a, int n, unsigned* mark, unsigned* sums, long long total,
-                        unsigned long long* count, cudaStream_t stream);
+cudaError_t launch_fuse(const FuseArgs& a, cudaStream_t stream);
+int fuse_tiles(int W, int H);  // blocks of the insertion for one keyframe
 cudaError_t launch_completeness(const CompletenessArgs& a, unsigned long long* count, cudaStream_t stream);
 cudaError_t launch_view_filter(const ViewFilterArgs& a, cudaStream_t stream);
 cudaError_t launch_project_kernel(int W, int H, int n, const float* dirs, float* uc, float* vc,
