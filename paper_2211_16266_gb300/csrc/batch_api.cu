@@ -238,11 +238,13 @@ static int build_plan(pmsp_ctx* c, BatchEngine& b, const pmsp_batch_item* items,
     c->stream = saved;
     if (rc) return rc;
     size_t flag_bytes = 0;
-    for (int i = 0; i < n; ++i) flag_bytes += ((size_t)plan.pixels[i] + 255) & ~size_t(255);
+    auto flags_of = [&](int i) { return (history_bytes(items[i].ref.w, items[i].ref.h, items[i].params.iterations) + 255) & ~size_t(255); };
+    for (int i = 0; i < n; ++i) flag_bytes += flags_of(i);
     if (uint8_t* flags = batch_flags(c, b, flag_bytes, st, b.capture && st == b.capture))
         for (int i = 0; i < n; ++i) {
-            plan.problems[i].changed = flags;
-            flags += ((size_t)plan.pixels[i] + 255) & ~size_t(255);
+            const cudaError_t e = bind_history(plan.problems[i], flags, items[i].params.iterations, st);
+            if (e != cudaSuccess) return cuda_fail(c, e, "batch history reset");
+            flags += flags_of(i);
         }
 
     // work lists: per phase, the tiles of every keyframe that has that phase

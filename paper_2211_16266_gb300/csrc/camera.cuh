@@ -186,6 +186,12 @@ __device__ __forceinline__ int wrap_index(int x, int W) {
     return x < 0 ? x + W : x;
 }
 
+// wrap_index for x at most 5 outside [0, W): without the division where W > 5.
+__device__ __forceinline__ int wrap_near(int x, int W) {
+    if (W <= 5) return wrap_index(x, W);
+    return x < 0 ? x + W : (x >= W ? x - W : x);
+}
+
 __device__ __forceinline__ int clamp_index(int x, int hi) { return x < 0 ? 0 : (x > hi ? hi : x); }
 
 }  // namespace pmsp

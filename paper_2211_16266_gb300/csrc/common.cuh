@@ -52,6 +52,7 @@ struct alignas(16) PixelParams {
     float* nz;
     float* cost;
     uint8_t* changed;     // W*H flags: the pixel's last half-sweep replaced its plane; NULL: no history
+    unsigned* close;      // per half-sweep of the run, its pixels that ended close; NULL: pooled half-sweeps only
     float d_min, d_max;
     float inv_dmin, inv_dmax;
     int S;                // number of sources

@@ -72,11 +72,59 @@ struct SweepPool {
 };
 struct NoPool {};
 
+// Further scratch of the bounded half-sweep (sweep_bounded): the bearing tables as
+// float2, the neighbours' FP32 bearings, each pixel's incumbent, how far a bound
+// must clear it, the random steps of its refinement tests (of the inverse range and
+// the normal, scaled), the costs of the tests under way, and the window's samples
+// in the order they are taken (the centre-most first, then row-major). MAX_DRAWN
+// tests are drawn ahead, the paper's six; further ones are drawn when they start.
+// At most MAX_AHEAD tests of a pixel are under way.
+constexpr int MAX_DRAWN = 6, MAX_AHEAD = 2;
+constexpr int MAX_REACH = 5;  // of a neighbour candidate (c_neighbors)
+// (Byte offsets in the reference tile and in the tables of float2 rows and
+// columns, and the spatial log2-weight: 16 bytes, or 8 where a window has many.)
+struct WindowSample {
+    int ref_at, row_at, col_at;
+    float wsp;
+    __device__ __forceinline__ static WindowSample at(int pitch, int dy, int dx, float wsp) {
+        return WindowSample{4 * (dy * pitch + dx), 8 * dy, 8 * dx, wsp};
+    }
+    __device__ __forceinline__ int ref() const { return ref_at; }
+    __device__ __forceinline__ int row() const { return row_at; }
+    __device__ __forceinline__ int col() const { return col_at; }
+};
+struct PackedSample {
+    short ref_at;
+    signed char dy, dx;
+    float wsp;
+    __device__ __forceinline__ static PackedSample at(int pitch, int dy, int dx, float wsp) {
+        return PackedSample{(short)(4 * (dy * pitch + dx)), (signed char)dy, (signed char)dx, wsp};
+    }
+    __device__ __forceinline__ int ref() const { return ref_at; }
+    __device__ __forceinline__ int row() const { return 8 * dy; }
+    __device__ __forceinline__ int col() const { return 8 * dx; }
+};
+template <int TW, int TH, int HALO, int SAMPLES>
+struct BoundPool {
+    static constexpr int N = (TW / 2) * TH;
+    float2 row[TH + 2 * HALO], col[TW + 2 * HALO];  // (cos, sin) latitude, (sin, cos) longitude of the tile
+    float2 near_row[TH + 2 * MAX_REACH], near_col[TW + 2 * MAX_REACH];  // (sin, cos), as pixel_bearing
+    float d[N], inv_d[N], nx[N], ny[N], nz[N], cost[N];
+    float margin[N];
+    float draw[MAX_DRAWN][4][N];
+    float result[MAX_AHEAD][N];
+    unsigned char version[N];  // counts the incumbents; a test of an older one is void
+    unsigned char taken[N];    // refinement results taken up
+    unsigned offer[BLOCK_THREADS];
+    using Sample = typename std::conditional<(SAMPLES <= 64), WindowSample, PackedSample>::type;
+    alignas(16) Sample sample[SAMPLES];
+};
+
 // Shared memory of one tile of TW x TH reference pixels with a halo of HALO
 // pixels on each side (the window radius the tile serves: the largest, or
 // that of a fixed-window instance); every shape has (TW / 2) x TH pixels of
 // one colour and TPP threads per pixel, 128 threads in all.
-template <int TW, int TH, int TPP = 1, int HALO = MAX_HALO, bool POOL = TPP == 1>
+template <int TW, int TH, int TPP = 1, int HALO = MAX_HALO, bool POOL = TPP == 1, bool BOUND = false>
 struct TileSmemT {
     static constexpr int W = TW, H = TH;
     static constexpr int PITCH = TW + 2 * HALO, ROWS = TH + 2 * HALO;
@@ -89,6 +137,9 @@ struct TileSmemT {
     float wsp[2 * HALO + 1];             // spatial log2-weight of offset index k
     // candidate pooling of the one-thread-per-pixel half-sweep
     typename std::conditional<POOL, SweepPool, NoPool>::type pool;
+    // the bounded half-sweep's (36 samples at 11x11 / 2, (2 HALO + 1)^2 at most)
+    static constexpr int SAMPLES = HALO == 5 ? 36 : (2 * HALO + 1) * (2 * HALO + 1);
+    typename std::conditional<BOUND, BoundPool<TW, TH, HALO, SAMPLES>, NoPool>::type bound;
 };
 using TileSmem = TileSmemT<TILE_W, TILE_H>;  // the batched and no-alloc kernels' shape
 
@@ -122,6 +173,11 @@ __device__ __forceinline__ auto& col_table() {
 // address, with the offsets in the instruction. Volatile, so that they are not
 // moved across a barrier.
 __device__ __forceinline__ unsigned shared_at(const void* p) { return (unsigned)__cvta_generic_to_shared(p); }
+__device__ __forceinline__ float shared_f(unsigned a) {
+    float v;
+    asm volatile("ld.shared.f32 %0, [%1];" : "=f"(v) : "r"(a));
+    return v;
+}
 template <int OFFSET = 0>
 __device__ __forceinline__ float2 shared_f2(unsigned a) {
     float2 v;
@@ -208,15 +264,17 @@ __device__ __forceinline__ float bilateral(const PixelParams& P, const SM& sm, i
 }
 
 // Local (halo-inclusive) tile coordinates of the pixel: lx, ly.
-template <class SM>
-__device__ __forceinline__ RefStats ref_stats(const PixelParams& P, const SM& sm, int lx, int ly) {
+// SII: sum w (I - mu)^2; w_centre: weight of the centre-most sample.
+template <int WIN, class SM>
+__device__ __forceinline__ RefStats ref_stats(const PixelParams& P, const SM& sm, int lx, int ly, float& SII,
+                                              float& w_centre) {
     RefStats st;
     st.Ip = sm.ref[ly * SM::PITCH + lx];
-    const int R = P.radius, stp = P.stride;
+    const int K = Window<WIN>::K(P), R = Window<WIN>::R(P), stp = Window<WIN>::stride(P);
     float Sw = 0.f, SI = 0.f;
-    for (int a = 0; a < P.K; ++a) {
+    for (int a = 0; a < K; ++a) {
         const float* row = sm.ref + (ly + a * stp - R) * SM::PITCH + lx - R;
-        for (int b = 0; b < P.K; ++b) {
+        for (int b = 0; b < K; ++b) {
             const float Iq = row[b * stp];
             const float w = bilateral(P, sm, a, b, Iq, st.Ip);
             Sw += w;
@@ -226,9 +284,9 @@ __device__ __forceinline__ RefStats ref_stats(const PixelParams& P, const SM& sm
     st.Sw = Sw;
     st.mu = SI / Sw;
     float SIc = 0.f, SIIc = 0.f;
-    for (int a = 0; a < P.K; ++a) {
+    for (int a = 0; a < K; ++a) {
         const float* row = sm.ref + (ly + a * stp - R) * SM::PITCH + lx - R;
-        for (int b = 0; b < P.K; ++b) {
+        for (int b = 0; b < K; ++b) {
             const float Iq = row[b * stp];
             const float w = bilateral(P, sm, a, b, Iq, st.Ip);
             const float Ic = Iq - st.mu;
@@ -238,7 +296,16 @@ __device__ __forceinline__ RefStats ref_stats(const PixelParams& P, const SM& sm
     }
     st.SIc = SIc;
     st.varI = mul_sub(Sw, SIIc, SIc, SIc);
+    SII = SIIc;
+    const int ac = K >> 1, o = ac * stp - R;
+    w_centre = bilateral(P, sm, ac, ac, sm.ref[(ly + o) * SM::PITCH + lx + o], st.Ip);
     return st;
+}
+
+template <class SM>
+__device__ __forceinline__ RefStats ref_stats(const PixelParams& P, const SM& sm, int lx, int ly) {
+    float SII, w_centre;
+    return ref_stats<0>(P, sm, lx, ly, SII, w_centre);
 }
 
 // Where the per-view constants are read from. Kernel parameters: plain member
@@ -380,6 +447,26 @@ __device__ __forceinline__ float view_sample(const SourceView& V, float X, float
     return sample_bilinear_half(L.tex(), L.inv_w(), L.inv_h(), qu, qv, front);
 }
 
+// Mean of the best_k smallest of NS view costs: odd-even transposition sort,
+// then the sum from the smallest up.
+template <int NS>
+__device__ __forceinline__ float best_mean(const PixelParams& P, float (&cs)[NS]) {
+#pragma unroll
+    for (int pass = 0; pass < NS; ++pass) {
+#pragma unroll
+        for (int s = (pass & 1); s + 1 < NS; s += 2) {
+            const float lo = fminf(cs[s], cs[s + 1]), hi = fmaxf(cs[s], cs[s + 1]);
+            cs[s] = lo;
+            cs[s + 1] = hi;
+        }
+    }
+    float sum = 0.f;
+#pragma unroll
+    for (int s = 0; s < NS; ++s)
+        if (s < P.best_k) sum += cs[s];
+    return sum / (float)P.best_k;
+}
+
 // Cost of plane (range d along rp, unit normal n) at the pixel. Returns 2 for
 // an invalid plane (a patch ray meets it from behind or grazing). NS views
 // are kept in registers; EXACT means S == NS (no per-view guard).
@@ -460,21 +547,7 @@ __device__ __forceinline__ float plane_cost(const PixelParams& P, const SM& sm, 
         }
         cs[s] = c;
     }
-    // odd-even transposition sort, then the mean of the best_k smallest
-#pragma unroll
-    for (int pass = 0; pass < NS; ++pass) {
-#pragma unroll
-        for (int s = (pass & 1); s + 1 < NS; s += 2) {
-            const float lo = fminf(cs[s], cs[s + 1]), hi = fmaxf(cs[s], cs[s + 1]);
-            cs[s] = lo;
-            cs[s + 1] = hi;
-        }
-    }
-    float sum = 0.f;
-#pragma unroll
-    for (int s = 0; s < NS; ++s)
-        if (s < P.best_k) sum += cs[s];
-    return sum / (float)P.best_k;
+    return best_mean<NS>(P, cs);
 }
 
 // Intensities of all NP view pairs (views 2q, 2q + 1) at the sample whose
@@ -501,15 +574,10 @@ __device__ __forceinline__ void pairs_columns(unsigned col, float2 (&U)[NP][3]) 
     }
 }
 
-template <int NP, class VA, int PITCH, bool AT_ADDRESS = false>
-__device__ __forceinline__ void pairs_sample(const PixelParams& P, float alpha, float beta, int cx, float2 (&J)[NP]) {
-    float2 U[NP][3];
-    if constexpr (AT_ADDRESS) {
-        pairs_columns<NP, PITCH>(shared_at(&col_table<NP, VA, PITCH>()[0][0][cx]), U);
-    } else {
-#pragma unroll
-        for (int k = 0; k < 3 * NP; ++k) U[k / 3][k % 3] = col_table<NP, VA, PITCH>()[k / 3][k % 3][cx];
-    }
+// The rest of pairs_sample, from the column's table entries U.
+template <int NP, class VA>
+__device__ __forceinline__ void pairs_sample_columns(const PixelParams& P, float alpha, float beta, const float2 (&U)[NP][3],
+                                                     float2 (&J)[NP]) {
     float2 fx[NP], fy[NP];
     float4 G0[NP], G1[NP];
     const float2 av = pair(alpha), bv = pair(beta);
@@ -549,6 +617,18 @@ __device__ __forceinline__ void pairs_sample(const PixelParams& P, float alpha, 
         const float top1 = fmaf(fx[q].y, g1.z - g1.w, g1.w), bot1 = fmaf(fx[q].y, g1.y - g1.x, g1.x);
         J[q] = make_float2(fmaf(fy[q].x, bot0 - top0, top0), fmaf(fy[q].y, bot1 - top1, top1));
     }
+}
+
+template <int NP, class VA, int PITCH, bool AT_ADDRESS = false>
+__device__ __forceinline__ void pairs_sample(const PixelParams& P, float alpha, float beta, int cx, float2 (&J)[NP]) {
+    float2 U[NP][3];
+    if constexpr (AT_ADDRESS) {
+        pairs_columns<NP, PITCH>(shared_at(&col_table<NP, VA, PITCH>()[0][0][cx]), U);
+    } else {
+#pragma unroll
+        for (int k = 0; k < 3 * NP; ++k) U[k / 3][k % 3] = col_table<NP, VA, PITCH>()[k / 3][k % 3][cx];
+    }
+    pairs_sample_columns<NP, VA>(P, alpha, beta, U, J);
 }
 
 // plane_cost for exactly NS >= 2 views held in kernel parameters, with the
@@ -644,20 +724,7 @@ __device__ __forceinline__ float plane_cost_paired(const PixelParams& P, const S
         cs[2 * q + 1] = view_cost(SJ[q].y, SJJ[q].y, SIJ[q].y);
     }
     if (ODD) cs[NS - 1] = view_cost(SJo, SJJo, SIJo);
-#pragma unroll
-    for (int pass = 0; pass < NS; ++pass) {
-#pragma unroll
-        for (int s = (pass & 1); s + 1 < NS; s += 2) {
-            const float lo = fminf(cs[s], cs[s + 1]), hi = fmaxf(cs[s], cs[s + 1]);
-            cs[s] = lo;
-            cs[s + 1] = hi;
-        }
-    }
-    float sum = 0.f;
-#pragma unroll
-    for (int s = 0; s < NS; ++s)
-        if (s < P.best_k) sum += cs[s];
-    return sum / (float)P.best_k;
+    return best_mean<NS>(P, cs);
 }
 
 // The paired form serves exactly known view counts whose views sit in kernel
@@ -741,6 +808,27 @@ __device__ __forceinline__ unsigned ordered_bits(float c) {
 }
 __device__ __forceinline__ float from_ordered_bits(unsigned o) {
     return __uint_as_float((o & 0x80000000u) ? (o & 0x7fffffffu) : ~o);
+}
+
+// View counts with a bounded half-sweep (launch_pixel_kernel_ns).
+constexpr bool has_bounded(int ns, bool exact) { return exact && ns >= 4 && ns <= 10; }
+
+// Pixels whose incumbent costs less than this: enough of a refinement test's samples
+// bound its cost above them.
+constexpr float CLOSE_COST = 0.15f;
+
+// Whether the half-sweep of (iter, colour) goes to the bounded kernel: half of the
+// pixels of the half-sweep before it ended close. Every half-sweep of such a run
+// is launched as both kernels, and one of them finds that it is not its turn.
+__device__ __forceinline__ bool bounded_turn(const PixelParams& P) {
+    const int phase = 2 * P.iter + P.colour;
+    return phase > 0 && P.close[phase - 1] >= (unsigned)((long long)P.W * P.H / 4);
+}
+
+// The half-sweep's close pixels, for the next one's choice (the block calls it).
+__device__ __forceinline__ void count_close(const PixelParams& P, bool close) {
+    const int n = __syncthreads_count(close);
+    if (threadIdx.x == 0 && n) atomicAdd(P.close + 2 * P.iter + P.colour, (unsigned)n);
 }
 
 // One half-sweep over the pixels of `colour` in a tile (Sec. III-C): each
@@ -880,6 +968,8 @@ __device__ __forceinline__ void sweep_pooled(const PixelParams& P, SM& sm, int b
         }
     }
     if (n_jobs == pooled_rounds) adopt_best();
+    if constexpr (has_bounded(NS, EXACT) && std::is_same<VA, ParamViews>::value)
+        if (P.close != nullptr) count_close(P, active && bc < CLOSE_COST);
     if (!active) return;
     if (P.changed) P.changed[i] = replaced;
     P.depth[i] = bd;
@@ -887,6 +977,507 @@ __device__ __forceinline__ void sweep_pooled(const PixelParams& P, SM& sm, int b
     P.ny[i] = bn.y;
     P.nz[i] = bn.z;
     P.cost[i] = bc;
+}
+
+// A refinement candidate's cost must fall below the incumbent's to matter, and
+// most end far above it. After part of the samples the cost is already bounded
+// from below: over the samples A taken so far let V_I, V_J and C be the weighted
+// variances and covariance; whatever the source shows at the others, the best it
+// can do is follow the reference exactly, J = a + b I, so with the residual
+// r = (V_I - C^2 / V_J) / Sw_A of the samples taken (V_I / Sw_A where C <= 0,
+// scaled sums as below) and the whole window's V = varI / Sw,
+//   NCC^2 <= V / (V + r),
+// and the cost is at least the mean of 1 - NCC over the best_k views of highest
+// bound. A candidate whose bound clears the incumbent is dropped; the others
+// are evaluated to the end by the same operations in the same order as ever, so
+// the maps do not change.
+//
+// Rounding: with n samples, u = 2^-24, A = Sw / w_c (w_c the weight of the
+// centre-most sample, on which every view is centred: varJ >= w_c sum w J^2, so
+// no sum of J cancels by more than A) and B = Sw sum w I^2 / varI, standard
+// forward error bounds on the sums give at most (6 n + 8) u A B for the computed
+// cost and (8 n + 9) u A B for the computed bound; refine_margin is their sum
+// plus a few roundings of the remaining operations. Where it is large (a
+// negligible centre weight, a flat patch) nothing is dropped.
+__device__ __forceinline__ float refine_margin(const RefStats& st, float SII, float wc, int n) {
+    const float AB = (st.Sw / wc) * (st.Sw * SII / st.varI);
+    const float m = fmaf(5.9604645e-8f * (float)(14 * n + 20), AB, 4e-6f);
+    return m < 0.1f ? m : __int_as_float(0x7f800000);
+}
+
+// Largest NCC a view can still reach (see above): V_I, V_J, C over the samples
+// taken, scaled by their weight; scale = Sw / (varI Sw_A); `whole`: all samples
+// are taken and the NCC itself is returned (0 where negative).
+__device__ __forceinline__ float ncc_bound(float VI, float VJ, float C, float scale, float floor_vj, bool whole) {
+    const float q = C > 0.f ? C * (C * rcp_approx(VJ)) : 0.f;
+    const float free = rcp_approx(fmaf(VI - q, scale, 1.0f));
+    const float m2 = whole ? q * rcp_approx(VI) : free;
+    return VJ > floor_vj ? sqrt_approx(m2) : 1.0f;
+}
+
+// The random steps of refinement test t (Sec. III-C item 1) of pixel i: of the
+// inverse range in x, of the normal in y, z, w, each 2^-(t+1) (2 u - 1), exact in
+// FP32.
+__device__ __forceinline__ U4 refinement_steps(const PixelParams& P, size_t i, int iter, int t) {
+    const float sc = __int_as_float((126 - t) << 23);  // 2^-(t+1)
+    U4 u = draw_uniform4((unsigned)i, (unsigned)iter, (unsigned)(1 + t), P.seed, P.keyframe);
+    u.x = (2.0f * u.x - 1.0f) * sc;
+    u.y = (2.0f * u.y - 1.0f) * sc;
+    u.z = (2.0f * u.z - 1.0f) * sc;
+    u.w = (2.0f * u.w - 1.0f) * sc;
+    return u;
+}
+
+// Refinement candidate t of pixel jt of the block, whose ray is rp and index in
+// the image i: its incumbent perturbed by the drawn steps.
+template <class SM>
+__device__ __forceinline__ void refinement_candidate(const PixelParams& P, const SM& sm, int jt, size_t i, int iter, int t,
+                                                     float3 rp, float& dc, float3& nc) {
+    U4 u;
+    if (t < MAX_DRAWN) {
+        u.x = sm.bound.draw[t][0][jt];
+        u.y = sm.bound.draw[t][1][jt];
+        u.z = sm.bound.draw[t][2][jt];
+        u.w = sm.bound.draw[t][3][jt];
+    } else {
+        u = refinement_steps(P, i, iter, t);
+    }
+    float inv = fmaf(u.x, P.inv_dmin - P.inv_dmax, sm.bound.inv_d[jt]);
+    inv = fminf(P.inv_dmin, fmaxf(P.inv_dmax, inv));
+    dc = 1.0f / inv;
+    nc = make_float3(__fadd_rn(u.y, sm.bound.nx[jt]), __fadd_rn(u.z, sm.bound.ny[jt]), __fadd_rn(u.w, sm.bound.nz[jt]));
+    const float il = 1.0f / sqrtf(dot3(nc, nc));
+    nc = face_camera(make_float3(nc.x * il, nc.y * il, nc.z * il), rp);
+}
+
+template <class SM>
+__device__ __forceinline__ void set_incumbent(SM& sm, int jt, float d, float3 n, float c) {
+    sm.bound.d[jt] = d;
+    sm.bound.inv_d[jt] = 1.0f / d;
+    sm.bound.nx[jt] = n.x;
+    sm.bound.ny[jt] = n.y;
+    sm.bound.nz[jt] = n.z;
+    sm.bound.cost[jt] = c;
+}
+
+// neighbour_candidate with the neighbour's bearing from the block's tables (the
+// same FP32 sines and cosines): pixel (x, y) of a tile at (bx, by).
+template <class SM>
+__device__ __forceinline__ bool neighbour_from_tables(const PixelParams& P, const SM& sm, int bx, int by, int x, int y,
+                                                      float3 rp, int k, float& dc, float3& nc) {
+    const int dx = c_neighbors[P.table][k][0], dy = c_neighbors[P.table][k][1];
+    const int qy = y + dy;
+    if (qy < 0 || qy >= P.H) return false;
+    const size_t j = (size_t)qy * P.W + wrap_near(x + dx, P.W);
+    nc = make_float3(P.nx[j], P.ny[j], P.nz[j]);
+    const float den = dot3(nc, rp);
+    const float2 r = sm.bound.near_row[qy - by + MAX_REACH], c = sm.bound.near_col[x + dx - bx + MAX_REACH];
+    const float3 rq = make_float3(r.y * c.x, -r.x, r.y * c.y);
+    dc = P.depth[j] * dot3(nc, rq) / den;
+    return den < -1e-6f && dc >= P.d_min && dc <= P.d_max;
+}
+
+// One half-sweep over the pixels of `colour` in a tile (Sec. III-C), for exactly
+// NS views: the maps of sweep_pooled bit for bit, by one loop that advances every
+// lane by K samples of its own candidate (a window has K x K).
+//
+// First the neighbour candidates of the warp's pixels, pooled, 32 at a time to
+// the end (their costs lie near the incumbent's: a bound drops almost none).
+// Then the refinement tests, each dropped as soon as it provably cannot win.
+// Dropped at different times, the tests leave lanes free, so any lane takes any
+// pixel's test: the next test of each pixel first, and where lanes are left over,
+// tests further ahead, on the supposition that those before them fail (on
+// converged maps 1 in 30 succeeds). The owner lane takes up a pixel's results in
+// order; a success makes the tests started from the older incumbent void, and
+// they are started again.
+//
+// Bound, like sweep_pooled, by FP32 issue of the samples taken (367 instructions a
+// sample of 6 views). On a converged 960x480 keyframe of 6 views a test is dropped
+// after 2.5 of 6 rows on average; lanes left idle and the hand-out keep a third of
+// that from the clock. 1920x960, 6 views, 8 iterations: 75.9 -> 66.8 ms; 4 views at
+// 960x480 14.7 -> 13.5 ms; 3840x1920, 8 views without noise, 4 iterations 229 ->
+// 206 ms. With sensor noise (costs around 0.4) the bound drops nothing and the hand-
+// out costs 6 %, so such half-sweeps stay with the pooled kernel (bounded_turn).
+template <int NS, class VA, int WIN, class SM>
+__device__ __forceinline__ void sweep_bounded(const PixelParams& P, SM& sm, int bx, int by, int colour, int iter) {
+    constexpr int NP = NS / 2, NPA = NP > 0 ? NP : 1;
+    constexpr bool ODD = (NS & 1) != 0;
+    using Sample = typename std::remove_reference<decltype(sm.bound)>::type::Sample;
+    constexpr int MIN_FREE = 8;  // lanes that are free before new tests are handed out
+    static_assert(SM::W / 2 * SM::H == BLOCK_THREADS, "a lane per pixel");
+    const int K = Window<WIN>::K(P), R = Window<WIN>::R(P), stp = Window<WIN>::stride(P);
+    const int ac = K >> 1;
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    const unsigned below = (1u << lane) - 1u;
+    // pixel jt of the block
+    auto pixel_x = [&](int jt, int py) { return bx + 2 * (jt % (SM::W / 2)) + ((py + colour) & 1); };
+    auto pixel_y = [&](int jt) { return by + jt / (SM::W / 2); };
+    auto pixel_ray = [&](int lx, int ly) {
+        return make_float3(sm.row_cos[ly] * sm.col_sin[lx], -sm.row_sin[ly], sm.row_cos[ly] * sm.col_cos[lx]);
+    };
+    const int own = threadIdx.x, oy = pixel_y(own), ox = pixel_x(own, oy);
+    const bool owner = ox < P.W && oy < P.H;
+    const size_t oi = (size_t)oy * P.W + ox;
+    unsigned need = 0;
+    for (int k = threadIdx.x; k < K * K; k += BLOCK_THREADS) {
+        const int centre = ac * K + ac, at = k == 0 ? centre : (k <= centre ? k - 1 : k);
+        const int a = at / K, b = at - a * K, dy = a * stp - R, dx = b * stp - R;
+        sm.bound.sample[k] = Sample::at(SM::PITCH, dy, dx, __fadd_rn(sm.wsp[a], sm.wsp[b]));
+    }
+    for (int k = threadIdx.x; k < SM::H + 2 * R; k += BLOCK_THREADS) sm.bound.row[k] = make_float2(sm.row_cos[k], sm.row_sin[k]);
+    for (int k = threadIdx.x; k < SM::W + 2 * R; k += BLOCK_THREADS) sm.bound.col[k] = make_float2(sm.col_sin[k], sm.col_cos[k]);
+    for (int k = threadIdx.x; k < SM::W + SM::H + 4 * MAX_REACH; k += BLOCK_THREADS) {
+        float sn, cs;  // the angles of pixel_bearing
+        if (k < SM::H + 2 * MAX_REACH) {
+            sincospif(0.5f - (2.0f * (by + k - MAX_REACH) + 1.0f) / (2.0f * P.H), &sn, &cs);
+            sm.bound.near_row[k] = make_float2(sn, cs);
+        } else {
+            const int c = k - (SM::H + 2 * MAX_REACH);
+            sincospif((2.0f * wrap_index(bx + c - MAX_REACH, P.W) + 1.0f) / P.W - 1.0f, &sn, &cs);
+            sm.bound.near_col[c] = make_float2(sn, cs);
+        }
+    }
+    __syncthreads();
+    if (owner) {
+        const int lx = ox - bx + R, ly = oy - by + R;
+        unsigned settled = 0;  // neighbours whose plane was tried in the last half-sweep
+        if (P.changed != nullptr && iter > 0) {
+#pragma unroll
+            for (int k = 0; k < 8; ++k) settled |= (unsigned)unchanged_neighbour(P, ox, oy, k) << k;
+        }
+        const float3 rp = pixel_ray(lx, ly);
+        float SII, w_centre;
+        const RefStats st = ref_stats<WIN>(P, sm, lx, ly, SII, w_centre);
+        sm.pool.st[own] = st;
+        sm.bound.margin[own] = refine_margin(st, SII, w_centre, K * K);
+        const float bd = P.depth[oi];
+        const float3 bn = make_float3(P.nx[oi], P.ny[oi], P.nz[oi]);
+        set_incumbent(sm, own, bd, bn, P.cost[oi]);
+        sm.bound.version[own] = 0;
+        sm.bound.taken[own] = 0;
+        sm.pool.key[own] = ~0ull;
+        float cd[8];
+        float3 cn[8];
+#pragma unroll
+        for (int k = 0; k < 8; ++k) {
+            const bool ok = neighbour_from_tables(P, sm, bx, by, ox, oy, rp, k, cd[k], cn[k]);
+            bool dup = same_plane(cd[k], cn[k], bd, bn);
+#pragma unroll
+            for (int m = 0; m < k; ++m) dup = dup || (((need >> m) & 1u) && same_plane(cd[k], cn[k], cd[m], cn[m]));
+            if (ok && !dup && !((settled >> k) & 1u)) need |= 1u << k;
+        }
+    }
+    const int n_refine = P.n_refine;
+    for (int t = 0; t < min(n_refine, MAX_DRAWN); ++t) {
+        const U4 u = refinement_steps(P, oi, iter, t);
+        sm.bound.draw[t][0][own] = u.x;
+        sm.bound.draw[t][1][own] = u.y;
+        sm.bound.draw[t][2][own] = u.z;
+        sm.bound.draw[t][3][own] = u.w;
+    }
+    // this lane's first slot in the warp's list: exclusive prefix of the counts
+    const int cnt = __popc(need);
+    int off = cnt;
+#pragma unroll
+    for (int d = 1; d < 32; d <<= 1) {
+        const int v = __shfl_up_sync(0xffffffffu, off, d);
+        if (lane >= d) off += v;
+    }
+    const int total = __shfl_sync(0xffffffffu, off, 31);
+    off -= cnt;
+    unsigned char* items = sm.pool.item[warp];
+    for (unsigned m = need; m; m &= m - 1) items[off++] = (unsigned char)((lane << 3) | (__ffs(m) - 1));
+    __syncthreads();  // the samples are listed by the whole block
+
+    bool pooled = total > 0, run = false, valid = false, replaced = false;
+    bool more = true, hit = false;   // (of the warp) tests not yet started; a test that beat the incumbent
+    int next = 0;                    // pooled: list position of the next candidates
+    int version = 0, taken = owner ? 0 : n_refine, issued = taken;  // the own pixel's incumbent; its tests: results taken up, started
+    int g = K;                       // groups of K samples taken of the current candidate
+    int jt = own, jk = 0, jv = 0;    // its pixel, its neighbour or test number, the version of its incumbent
+    int lx = R, ly = R;              // the pixel's place in the tile
+    float dc = 0.f, dn = 0.f, Ip = 0.f, mu = 0.f;
+    float3 nc = make_float3(0.f, 0.f, 0.f);
+    float2 c0[NPA], SJ[NPA], SJJ[NPA], SIJ[NPA];
+    float c0o = 0.f, SJo = 0.f, SJJo = 0.f, SIJo = 0.f;
+    float sw = 0.f, sI = 0.f, sII = 0.f;  // the reference's sums over the samples taken
+#pragma unroll
+    for (int q = 0; q < NPA; ++q) c0[q] = SJ[q] = SJJ[q] = SIJ[q] = pair(0.f);
+    for (;;) {
+        // new candidates: pooled, for the whole warp; then, for the lanes that are free
+        const unsigned resting = __ballot_sync(0xffffffffu, !run);
+        if (pooled ? g == K : resting == 0xffffffffu || hit || (more && __popc(resting) >= MIN_FREE)) {
+            bool job = false;
+            if (pooled && next >= total) {  // every neighbour candidate has been scored
+                __syncwarp();
+                if (owner) {
+                    const unsigned long long key = sm.pool.key[own];
+                    const float c = from_ordered_bits((unsigned)(key >> 3));
+                    if (key != ~0ull && c < sm.bound.cost[own]) {
+                        neighbour_from_tables(P, sm, bx, by, ox, oy, pixel_ray(ox - bx + R, oy - by + R), (int)(key & 7u), dc, nc);
+                        set_incumbent(sm, own, dc, nc, c);
+                        replaced = true;
+                    }
+                }
+                pooled = false;
+                run = false;
+            }
+            if (pooled) {
+                if (next + lane < total) {
+                    const int it = items[next + lane];
+                    jk = it & 7;
+                    jt = (warp << 5) + (it >> 3);
+                    job = true;
+                }
+                next += 32;
+            } else {
+                __syncwarp();
+                // take up the results of the own pixel's tests, in order (one that won when
+                // its turn had come has replaced the incumbent already)
+                if (owner && sm.bound.version[own] != version) {
+                    version = sm.bound.version[own];
+                    issued = taken = sm.bound.taken[own];
+                    replaced = true;
+                }
+                while (taken < issued) {
+                    const float c = sm.bound.result[taken % MAX_AHEAD][own];
+                    if (__float_as_uint(c) == 0xffffffffu) break;  // under way
+                    if (c < sm.bound.cost[own]) {
+                        float d;
+                        float3 n;
+                        refinement_candidate(P, sm, own, oi, iter, taken, pixel_ray(ox - bx + R, oy - by + R), d, n);
+                        set_incumbent(sm, own, d, n, c);
+                        sm.bound.version[own] = (unsigned char)++version;
+                        replaced = true;
+                        issued = taken + 1;
+                    }
+                    ++taken;
+                }
+                if (owner) sm.bound.taken[own] = (unsigned char)taken;
+                __syncwarp();
+                if (run && jv != sm.bound.version[jt]) run = false;
+                // hand out the pixels' next tests, then the ones after them
+                unsigned idle = __ballot_sync(0xffffffffu, !run);
+                for (int ahead = 0; ahead < MAX_AHEAD && idle != 0; ++ahead) {
+                    const bool offer = issued < n_refine && issued - taken == ahead;
+                    const unsigned m = __ballot_sync(0xffffffffu, offer);
+                    if (m == 0) continue;
+                    const int n_given = min(__popc(m), __popc(idle));
+                    const int rank = __popc(m & below);
+                    if (offer && rank < n_given) {
+                        sm.bound.offer[warp * 32 + rank] = (unsigned)(own | (issued << 8) | (version << 16));
+                        sm.bound.result[issued % MAX_AHEAD][own] = __uint_as_float(0xffffffffu);
+                        ++issued;
+                    }
+                    __syncwarp();
+                    const int at = __popc(idle & below);
+                    if (((idle >> lane) & 1u) && at < n_given) {
+                        const unsigned o = sm.bound.offer[warp * 32 + at];
+                        jt = (int)(o & 255u);
+                        jk = (int)((o >> 8) & 255u);
+                        jv = (int)(o >> 16);
+                        job = true;
+                    }
+                    __syncwarp();
+                    idle = __ballot_sync(0xffffffffu, !run && !job);
+                }
+                more = __any_sync(0xffffffffu, issued < n_refine);
+                hit = false;
+            }
+            if (job) {
+                const int jy = pixel_y(jt), jx = pixel_x(jt, jy);
+                lx = jx - bx + R;
+                ly = jy - by + R;
+                const float3 rp = pixel_ray(lx, ly);
+                if (pooled)
+                    neighbour_from_tables(P, sm, bx, by, jx, jy, rp, jk, dc, nc);
+                else
+                    refinement_candidate(P, sm, jt, (size_t)jy * P.W + jx, iter, jk, rp, dc, nc);
+                dn = dc * dot3(nc, rp);
+                const RefStats& st = sm.pool.st[jt];
+                Ip = st.Ip;
+                mu = st.mu;
+                valid = !(st.varI < 1e-8f * st.Sw * st.Sw);
+#pragma unroll
+                for (int q = 0; q < NPA; ++q) SJ[q] = SJJ[q] = SIJ[q] = pair(0.f);
+                SJo = SJJo = SIJo = sw = sI = sII = 0.f;
+            }
+            if (job || pooled) {
+                run = job;
+                g = 0;
+            }
+        }
+        if (!__any_sync(0xffffffffu, run)) break;
+        if (run) {
+            const unsigned ref = shared_at(sm.ref + ly * SM::PITCH + lx);
+            const unsigned row = shared_at(sm.bound.row + ly), col = shared_at(sm.bound.col + lx);
+            unsigned table = 0;  // from a column's bearing to its entry of the column table
+            if constexpr (NP > 0) table = shared_at(&col_table<NP, VA, SM::PITCH>()[0][0][0]) - shared_at(sm.bound.col);
+            const Sample* smp = sm.bound.sample + g * K;
+#pragma unroll 1
+            for (int j = 0; j < K; ++j) {
+                const Sample q = smp[j];
+                const float Iq = shared_f(ref + q.ref());
+                const float dI = Iq - Ip;
+                const float w = exp2_approx(fmaf(P.wc, dI * dI, q.wsp));
+                const float Ic = Iq - mu, wI = w * Ic;
+                const unsigned at = col + q.col();
+                const float2 rw = shared_f2(row + q.row()), cl = shared_f2(at);  // (cos, sin) latitude, (sin, cos) longitude
+                const float3 rq = make_float3(rw.x * cl.x, -rw.y, rw.x * cl.y);
+                const float den = dot3(nc, rq);
+                valid = valid && (den < -1e-6f);
+                const float t = __fdividef(dn, den);
+                float2 J[NPA];
+                if constexpr (NP > 0) {
+                    float2 U[NP][3];
+                    pairs_columns<NP, SM::PITCH>(at + table, U);
+                    pairs_sample_columns<NP, VA>(P, t * rw.x, t * rq.y, U, J);
+                }
+                float Jo = 0.f;
+                if (ODD) Jo = view_sample<VA>(P.src[NS - 1], t * rq.x, t * rq.y, t * rq.z);
+                if (j == 0) {  // the first sample of all centres every view
+                    if (g == 0) {
+#pragma unroll
+                        for (int p = 0; p < NP; ++p) c0[p] = J[p];
+                        c0o = Jo;
+                    }
+                }
+                const float2 w2 = pair(w), wI2 = pair(wI);
+                sw += w;
+                sI += wI;
+                sII = fmaf(wI, Ic, sII);
+#pragma unroll
+                for (int p = 0; p < NP; ++p) {
+                    const float2 Jc = add2(J[p], make_float2(-c0[p].x, -c0[p].y));
+                    const float2 tw = mul2(w2, Jc);
+                    SJ[p] = add2(SJ[p], tw);
+                    SJJ[p] = fma2(tw, Jc, SJJ[p]);
+                    SIJ[p] = fma2(wI2, Jc, SIJ[p]);
+                }
+                if (ODD) {
+                    const float Jc = Jo - c0o;
+                    const float tw = __fmul_rn(w, Jc);
+                    SJo = __fadd_rn(SJo, tw);
+                    SJJo = fmaf(tw, Jc, SJJo);
+                    SIJo = fmaf(wI, Jc, SIJo);
+                }
+            }
+        }
+        ++g;
+        bool done = run && g == K, dropped = false, won = false, in_turn = false;
+        float c_won = 0.f;
+        if (!pooled) {
+            float thr = 0.f, VI = 0.f, scale = 0.f;
+            bool may = false;
+            // (where half the warp ends at once, their costs come cheaper than a bound first)
+            const bool few = __popc(__ballot_sync(0xffffffffu, done)) < 16;
+            if (run) {
+                done = done || !valid;
+                const RefStats& st = sm.pool.st[jt];
+                thr = sm.bound.cost[jt] + sm.bound.margin[jt];
+                VI = fmaf(sw, sII, -(sI * sI));
+                scale = st.Sw * rcp_approx(st.varI * sw);
+                // were no view to correlate in the samples taken: the most the bound can be
+                may = valid && (g == K ? few : 1.0f - rsqrtf(fmaf(VI, scale, 1.0f)) > thr);
+            }
+            if (may) {
+                const float fl = 1e-8f * sw * sw;
+                float cs[NS];
+#pragma unroll
+                for (int p = 0; p < NP; ++p) {
+                    const float2 sw2 = pair(sw), sI2 = pair(-sI);
+                    const float2 VJ = fma2(sw2, SJJ[p], mul2(make_float2(-SJ[p].x, -SJ[p].y), SJ[p]));
+                    const float2 C = fma2(sw2, SIJ[p], mul2(sI2, SJ[p]));
+                    cs[2 * p] = ncc_bound(VI, VJ.x, C.x, scale, fl, g == K);
+                    cs[2 * p + 1] = ncc_bound(VI, VJ.y, C.y, scale, fl, g == K);
+                }
+                if (ODD) cs[NS - 1] = ncc_bound(VI, fmaf(sw, SJJo, -SJo * SJo), fmaf(sw, SIJo, -sI * SJo), scale, fl, g == K);
+                // the best_k largest, bubbled to the end one by one
+                float sum = 0.f;
+#pragma unroll
+                for (int b = 0; b < NS; ++b) {
+                    if (b >= P.best_k) break;
+#pragma unroll
+                    for (int q = 0; q + 1 < NS - b; ++q) {
+                        const float lo = fminf(cs[q], cs[q + 1]), hi = fmaxf(cs[q], cs[q + 1]);
+                        cs[q] = lo;
+                        cs[q + 1] = hi;
+                    }
+                    sum += 1.0f - cs[NS - 1 - b];
+                }
+                dropped = sum > thr * (float)P.best_k;
+            }
+            if (dropped) {
+                sm.bound.result[jk % MAX_AHEAD][jt] = 4.0f;  // no cost: above every one
+                done = run = false;
+            }
+        }
+        if (done) {
+            const RefStats& st = sm.pool.st[jt];
+            float c = 2.0f;
+            if (valid) {
+                const float eps = 1e-8f * st.Sw * st.Sw;
+                float cs[NS];
+                auto view_cost = [&](float sj, float sjj, float sij) {
+                    const float varJ = mul_sub(st.Sw, sjj, sj, sj);
+                    const float cov = mul_sub(st.Sw, sij, st.SIc, sj);
+                    if (varJ < eps) return 2.0f;
+                    float ncc = cov * rsqrtf(st.varI * varJ);
+                    ncc = fminf(1.0f, fmaxf(-1.0f, ncc));
+                    return 1.0f - ncc;
+                };
+#pragma unroll
+                for (int p = 0; p < NP; ++p) {
+                    cs[2 * p] = view_cost(SJ[p].x, SJJ[p].x, SIJ[p].x);
+                    cs[2 * p + 1] = view_cost(SJ[p].y, SJJ[p].y, SIJ[p].y);
+                }
+                if (ODD) cs[NS - 1] = view_cost(SJo, SJJo, SIJo);
+                c = best_mean<NS>(P, cs);
+            }
+            if (pooled) {
+                if (c == c) atomicMin(&sm.pool.key[jt], ((unsigned long long)ordered_bits(c) << 3) | (unsigned)jk);
+            } else {
+                sm.bound.result[jk % MAX_AHEAD][jt] = c;
+                run = false;
+                won = c < sm.bound.cost[jt];
+                in_turn = won && jk == sm.bound.taken[jt];
+                c_won = c;
+            }
+        }
+        if (!pooled && __any_sync(0xffffffffu, won)) {
+            hit = true;
+            __syncwarp();  // (every lane has seen whose turn it is)
+            if (in_turn) {
+                set_incumbent(sm, jt, dc, nc, c_won);
+                ++sm.bound.version[jt];
+                ++sm.bound.taken[jt];
+            }
+        }
+    }
+    count_close(P, owner && sm.bound.cost[own] < CLOSE_COST);
+    if (!owner) return;
+    P.changed[oi] = replaced;
+    if (!replaced) return;  // the planes stay as they are
+    P.depth[oi] = sm.bound.d[own];
+    P.nx[oi] = sm.bound.nx[own];
+    P.ny[oi] = sm.bound.ny[own];
+    P.nz[oi] = sm.bound.nz[own];
+    P.cost[oi] = sm.bound.cost[own];
+}
+
+// The tile's column table (see col_table), from its staged bearings.
+template <int NP, class VA, class SM>
+__device__ __forceinline__ void build_col_table(const PixelParams& P, const SM& sm) {
+    static_assert(NP <= PMSP_MAX_SOURCES / 2, "column table too small");
+    const int cols = SM::W + 2 * P.radius;
+    for (int i = threadIdx.x; i < cols * NP; i += BLOCK_THREADS) {
+        const int q = i / cols, c = i - q * cols;
+        const PixelParams::ViewPair& VP = P.pairs[q];
+        const float2 sn = pair(sm.col_sin[c]), cs = pair(sm.col_cos[c]);
+        col_table<NP, VA, SM::PITCH>()[q][0][c] = fma2(VP.R[0], sn, mul2(VP.R[2], cs));
+        col_table<NP, VA, SM::PITCH>()[q][1][c] = fma2(VP.R[3], sn, mul2(VP.R[5], cs));
+        col_table<NP, VA, SM::PITCH>()[q][2][c] = fma2(VP.R[6], sn, mul2(VP.R[8], cs));
+    }
 }
 
 // One tile of one problem: stage the reference tile, then every active
@@ -898,17 +1489,7 @@ __device__ __forceinline__ void process_tile(const PixelParams& P, SM& sm, int b
     stage_tile(P, sm, bx, by);
     __syncthreads();
     if constexpr (EXACT && NS >= 2 && paired_views<VA>()) {
-        constexpr int NP = NS / 2;
-        static_assert(NP <= PMSP_MAX_SOURCES / 2, "column table too small");
-        const int cols = SM::W + 2 * P.radius;
-        for (int i = threadIdx.x; i < cols * NP; i += BLOCK_THREADS) {
-            const int q = i / cols, c = i - q * cols;
-            const PixelParams::ViewPair& VP = P.pairs[q];
-            const float2 sn = pair(sm.col_sin[c]), cs = pair(sm.col_cos[c]);
-            col_table<NP, VA, SM::PITCH>()[q][0][c] = fma2(VP.R[0], sn, mul2(VP.R[2], cs));
-            col_table<NP, VA, SM::PITCH>()[q][1][c] = fma2(VP.R[3], sn, mul2(VP.R[5], cs));
-            col_table<NP, VA, SM::PITCH>()[q][2][c] = fma2(VP.R[6], sn, mul2(VP.R[8], cs));
-        }
+        build_col_table<NS / 2, VA>(P, sm);
         __syncthreads();
     }
 
@@ -948,7 +1529,24 @@ __global__ void __launch_bounds__(BLOCK_THREADS, pixel_min_blocks(NS)) pixel_ker
     __shared__ SM sm;
     int tx, ty;
     tile_of_block(gridDim.x, gridDim.y, blockIdx.y * gridDim.x + blockIdx.x, tx, ty);
+    if (MODE == MODE_SWEEP && has_bounded(NS, EXACT) && TS == 0 && P.close != nullptr && bounded_turn(P)) return;
     process_tile<NS, EXACT, MODE, ParamViews, WIN, SM>(P, sm, tx * SM::W, ty * SM::H, P.colour, P.iter);
+}
+
+// The bounded half-sweep of one tile (sweep_bounded), where it is its turn.
+template <int NS, int WIN>
+__global__ void __launch_bounds__(BLOCK_THREADS, pixel_min_blocks(NS)) bounded_kernel(const __grid_constant__ PixelParams P) {
+    using SM = TileSmemT<32, 8, 1, Window<WIN>::HALO, true, true>;
+    __shared__ SM sm;
+    if (!bounded_turn(P)) return;
+    int tx, ty;
+    tile_of_block(gridDim.x, gridDim.y, blockIdx.y * gridDim.x + blockIdx.x, tx, ty);
+    const int bx = tx * SM::W, by = ty * SM::H;
+    stage_tile(P, sm, bx, by);
+    __syncthreads();
+    build_col_table<NS / 2, ParamViews>(P, sm);
+    __syncthreads();
+    sweep_bounded<NS, ParamViews, WIN, SM>(P, sm, bx, by, P.colour, P.iter);
 }
 
 // Grid of a tile shape over a W x H panorama.
@@ -987,13 +1585,23 @@ inline void launch_tiles(const PixelParams& p, cudaStream_t stream) {
     pixel_kernel<NS, EXACT, MODE, WIN, TS><<<tile_grid<TS>(p), BLOCK_THREADS, 0, stream>>>(p);
 }
 
+// The bounded kernel's launch beside the pooled one's (see bounded_turn).
+template <int NS, bool EXACT, int WIN>
+inline void launch_bounded(const PixelParams& p, cudaStream_t stream) {
+    if constexpr (has_bounded(NS, EXACT)) {
+        if (p.close == nullptr || (p.iter == 0 && p.colour == 0)) return;
+        prefer_texture_cache<bounded_kernel<NS, WIN>>();
+        bounded_kernel<NS, WIN><<<tile_grid<0>(p), BLOCK_THREADS, 0, stream>>>(p);
+    }
+}
+
 // A fixed-window sweep in the problem's tile shape.
 template <int NS, bool EXACT, int WIN>
 inline void launch_sweep_window(const PixelParams& p, cudaStream_t stream) {
     switch (p.tile) {
         case 1: launch_tiles<NS, EXACT, MODE_SWEEP, WIN, 1>(p, stream); break;
         case 2: launch_tiles<NS, EXACT, MODE_SWEEP, WIN, 2>(p, stream); break;
-        default: launch_tiles<NS, EXACT, MODE_SWEEP, WIN, 0>(p, stream); break;
+        default: launch_tiles<NS, EXACT, MODE_SWEEP, WIN, 0>(p, stream); launch_bounded<NS, EXACT, WIN>(p, stream); break;
     }
 }
 
@@ -1037,6 +1645,7 @@ cudaError_t launch_pixel_kernel_ns(const PixelParams& p, int mode, cudaStream_t 
                 }
             }
             launch_tiles<NS, EXACT, MODE_SWEEP>(p, stream);
+            launch_bounded<NS, EXACT, 0>(p, stream);
             break;
     }
     return cudaGetLastError();

@@ -40,6 +40,8 @@ int check_maps(pmsp_ctx* c, const pmsp_maps* m, int W, int H, bool need_normal, 
 int ensure_buffer(pmsp_ctx* c, DevBuffer& b, size_t bytes);
 bool recording(cudaStream_t st);  // being captured (or not to be asked about it)
 uint8_t* change_flags(pmsp_ctx* c, size_t n);
+size_t history_bytes(int W, int H, int iterations);
+cudaError_t bind_history(PixelParams& P, uint8_t* mem, int iterations, cudaStream_t st);
 int upload_texture(pmsp_ctx* c, TexImage& t, const pmsp_image* im, cudaStream_t st);
 void free_texture(TexImage& t);
 void compose_rel(const pmsp_pose& r, const pmsp_pose& s, double R[9], double t[3]);

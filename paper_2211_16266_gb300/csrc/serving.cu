@@ -189,7 +189,8 @@ void fill_request(Serving& s, Request* r) {
     r->prob.ny = base + 2 * N;
     r->prob.nz = base + 3 * N;
     r->prob.cost = base + 4 * N;
-    r->prob.changed = reinterpret_cast<uint8_t*>(base + 5 * N);  // the filtered-depth plane, written only by the tail
+    // history in the filtered-depth plane, which only the tail writes (a lane zeroes its counters before the first sweep)
+    r->prob.changed = reinterpret_cast<uint8_t*>(base + 5 * N);
     r->prob.err = s.ctx->d_err;
 }
 
@@ -245,6 +246,8 @@ int enqueue_tail(Serving& s, Request* r, cudaStream_t st) {
 int enqueue_request(Serving& s, Request* r, cudaStream_t st) {
     PixelParams P = r->prob;
     cudaError_t e = cudaSuccess;
+    if (history_bytes(r->W, r->H, r->params.iterations) <= (size_t)r->W * r->H * sizeof(float))
+        e = bind_history(P, P.changed, r->params.iterations, st);
     for (int ph = 0; ph < r->n_phases && e == cudaSuccess; ++ph) {
         P.colour = ph & 1;
         P.iter = ph < 2 ? 0 : (ph - 2) >> 1;

@@ -1,7 +1,8 @@
 """Whole runs against the same run driven step by step, bit for bit.
 
 Within a run the half-sweeps leave out neighbour candidates that were already
-tried (PixelParams::changed); a half-sweep called on its own has no history and
+tried (PixelParams::changed), and on larger keyframes drop refinement tests that
+provably cannot win (sweep_bounded); a half-sweep called on its own has no history and
 tries them all. Both must give the same maps: in one call, warped, batched by
 either strategy, replayed from a graph, and recorded by the caller.
 """
@@ -25,14 +26,18 @@ FORMS = [  # W, H, views, format, window, stride, table, best_k, n_refine
     (96, 48, 1, "u8", 11, 2, 0, 1, 6), (66, 34, 2, "f16", 7, 1, 1, 1, 6), (250, 130, 3, "f32", 9, 3, 1, 2, 6),
     (8, 4, 2, "u8", 5, 1, 0, 2, 6), (128, 64, 6, "u8", 11, 2, 0, 3, 6), (100, 52, 7, "f32", 11, 2, 1, 7, 0),
     (64, 34, 10, "f16", 5, 2, 0, 4, 9), (64, 32, 12, "u8", 3, 1, 0, 3, 2), (70, 36, 16, "u8", 21, 5, 0, 16, 1),
+    # from 456 tiles on: the refinement tests dropped by a bound, in every window class, ragged, with more tests
+    # than are drawn ahead, with none, with no bilateral weights and with the mean over all views
+    (518, 250, 4, "u8", 11, 2, 0, 1, 6), (512, 256, 5, "f16", 7, 1, 1, 5, 9), (640, 200, 6, "f32", 9, 3, 0, 3, 6),
+    (514, 258, 7, "u8", 11, 2, 1, 2, 0), (512, 260, 10, "u8", 11, 2, 0, 3, 30),
 ]
 
 
 def _problem(form, n_iter):
     W, H, S, fmt, pw, st, table, k, nr = form
     p = scenes.trajectory_problem(W, H, S, seed_scene=1020 + S, fmt=fmt)
-    params = dict(d_min=0.3, d_max=10.0, patch_w=pw, patch_stride=st, iterations=n_iter, best_k=k, sigma_color=0.2,
-                  sigma_space=3.0, n_refine=nr, neighbor_table=table, seed=9, keyframe_id=S)
+    params = dict(d_min=0.3, d_max=10.0, patch_w=pw, patch_stride=st, iterations=n_iter, best_k=k,
+                  sigma_color=0.0 if S == 5 else 0.2, sigma_space=0.0 if S == 5 else 3.0, n_refine=nr, neighbor_table=table, seed=9, keyframe_id=S)
     import torch
     d = lambda a: torch.from_numpy(np.ascontiguousarray(a)).cuda()  # noqa: E731
     return (d(p.ref.image), (p.ref.R, p.ref.t), [d(f.image) for f in p.srcs], [(f.R, f.t) for f in p.srcs]), params
@@ -72,7 +77,7 @@ def test_run_equals_its_steps(pm, form):
 
 def test_batches_equal_their_steps(pm):
     import torch
-    probs = [_problem(FORMS[k], 3 + k % 3) for k in (0, 2, 4, 5, 6)]
+    probs = [_problem(FORMS[k], 3 + k % 3) for k in (0, 2, 4, 5, 6, 9, 12)]
     with pm.Context(0) as ctx:
         want = [_steps(pm, ctx, *p) for p in probs]
         for strategy in (0, 1):
