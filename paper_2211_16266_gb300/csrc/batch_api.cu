@@ -335,6 +335,7 @@ static int enqueue_branches(pmsp_ctx* c, BatchEngine& b, const BatchPlan& plan, 
         load[k] += plan.pixels[i] * plan.n_phases[i];
         PixelParams P = plan.problems[i];
         for (int ph = 0; ph < plan.n_phases[i] && e == cudaSuccess; ++ph) {
+            if (ph == 1) continue;  // the initialisation serves both colours in one launch
             P.colour = ph & 1;
             P.iter = ph < 2 ? 0 : (ph - 2) >> 1;
             e = launch_pixel_kernel(P, ph < 2 ? MODE_INIT : MODE_SWEEP, b.branch[k]);

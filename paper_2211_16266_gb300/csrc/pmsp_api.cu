@@ -23,7 +23,7 @@ template <int NS, bool EXACT>
 cudaError_t launch_pixel_kernel_ns(const PixelParams& p, int mode, cudaStream_t stream);
 
 // One instantiation per source count 1..16 (views unrolled without guards,
-// in packed pairs from 2 views on).
+// in packed pairs from 2 views on). MODE_INIT and MODE_COST serve both colours.
 cudaError_t launch_pixel_kernel(const PixelParams& p, int mode, cudaStream_t stream) {
     switch (p.S) {
         case 1: return launch_pixel_kernel_ns<1, true>(p, mode, stream);
@@ -506,10 +506,7 @@ int pmsp_densify(pmsp_ctx* c, const pmsp_image* ref, const pmsp_pose* ref_pose, 
     if (rc) return rc;
     if ((rc = check_maps(c, out, ref->w, ref->h, true, true, "output"))) return rc;
     if ((rc = bind_maps(c, out, P, false))) return rc;
-    for (int colour = 0; colour < 2; ++colour) {
-        P.colour = colour;
-        if ((rc = launch(c, P, MODE_INIT))) return rc;
-    }
+    if ((rc = launch(c, P, MODE_INIT))) return rc;
     if (p->iterations > 0) {
         const cudaError_t e = bind_history(P, change_flags(c, history_bytes(P.W, P.H, p->iterations)), p->iterations, c->stream);
         if (e != cudaSuccess) return cuda_fail(c, e, "history reset");
@@ -567,10 +564,7 @@ static int warp_init_into(pmsp_ctx* c, PixelParams& P, const pmsp_maps* prev, co
     A.src = src;
     cudaError_t e = launch_warp_init(P, A, c->stream);
     if (e != cudaSuccess) return cuda_fail(c, e, "warp launch");
-    for (int colour = 0; colour < 2; ++colour) {
-        P.colour = colour;
-        if ((rc = launch(c, P, MODE_COST))) return rc;
-    }
+    if ((rc = launch(c, P, MODE_COST))) return rc;
     return PMSP_OK;
 }
 
@@ -625,10 +619,7 @@ int pmsp_cost_map(pmsp_ctx* c, const pmsp_image* ref, const pmsp_pose* ref_pose,
     if (rc) return rc;
     if ((rc = check_maps(c, planes, ref->w, ref->h, true, true, "planes"))) return rc;
     if ((rc = bind_maps(c, planes, P, true))) return rc;
-    for (int colour = 0; colour < 2; ++colour) {
-        P.colour = colour;
-        if ((rc = launch(c, P, MODE_COST))) return rc;
-    }
+    if ((rc = launch(c, P, MODE_COST))) return rc;
     return finish_maps(c, planes, P, false);
 }
 
@@ -641,10 +632,7 @@ int pmsp_init(pmsp_ctx* c, const pmsp_image* ref, const pmsp_pose* ref_pose, con
     if (rc) return rc;
     if ((rc = check_maps(c, out, ref->w, ref->h, true, true, "output"))) return rc;
     if ((rc = bind_maps(c, out, P, false))) return rc;
-    for (int colour = 0; colour < 2; ++colour) {
-        P.colour = colour;
-        if ((rc = launch(c, P, MODE_INIT))) return rc;
-    }
+    if ((rc = launch(c, P, MODE_INIT))) return rc;
     return finish_maps(c, out, P, true);
 }
 

@@ -249,6 +249,7 @@ int enqueue_request(Serving& s, Request* r, cudaStream_t st) {
     if (history_bytes(r->W, r->H, r->params.iterations) <= (size_t)r->W * r->H * sizeof(float))
         e = bind_history(P, P.changed, r->params.iterations, st);
     for (int ph = 0; ph < r->n_phases && e == cudaSuccess; ++ph) {
+        if (ph == 1) continue;  // the initialisation serves both colours in one launch
         P.colour = ph & 1;
         P.iter = ph < 2 ? 0 : (ph - 2) >> 1;
         e = launch_pixel_kernel(P, ph < 2 ? MODE_INIT : MODE_SWEEP, st);
