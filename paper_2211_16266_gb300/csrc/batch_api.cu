@@ -237,6 +237,10 @@ static int build_plan(pmsp_ctx* c, BatchEngine& b, const pmsp_batch_item* items,
     }
     c->stream = saved;
     if (rc) return rc;
+    auto tiles_of = [&](int i) { return (int64_t)((items[i].ref.w + TILE_W - 1) / TILE_W) * ((items[i].ref.h + TILE_H - 1) / TILE_H); };
+    int64_t tiles = 0;
+    for (int i = 0; i < n; ++i) tiles += tiles_of(i);
+    for (int i = 0; i < n; ++i) plan.problems[i].crowd = (int)std::min<int64_t>(tiles - tiles_of(i), 1 << 24);
     size_t flag_bytes = 0;
     auto flags_of = [&](int i) { return (history_bytes(items[i].ref.w, items[i].ref.h, items[i].params.iterations) + 255) & ~size_t(255); };
     for (int i = 0; i < n; ++i) flag_bytes += flags_of(i);

@@ -12,6 +12,7 @@ namespace pmsp {
 // Tile of reference pixels handled by one block: TILE_W x TILE_H pixels, of
 // which one colour (half of them) is active in a half-sweep; one thread per
 // active pixel.
+constexpr int SM_COUNT = 152;  // GB300; launch shapes are chosen by it
 constexpr int TILE_W = 32;
 constexpr int TILE_H = 8;
 constexpr int BLOCK_THREADS = (TILE_W / 2) * TILE_H;
@@ -67,6 +68,7 @@ struct alignas(16) PixelParams {
     unsigned long long seed, keyframe;
     int phase;            // batched serving: 0,1 initialisation colours, 2 + 2 t + c half-sweep (t, c)
     int tile;             // tile shape of the single-keyframe half-sweep: 0 32x8, 1 64x4, 2 16x16
+    int crowd;            // tiles of the keyframes that run beside this one
     int tpp;              // threads per pixel of the single-keyframe half-sweep: 1; 2 or 4 warps
                           // (views split); -2, -4 or -8: adjacent lanes (patch samples split)
     int colour;

@@ -61,14 +61,15 @@ struct RefStats {
     float varI;  // Sw * sum w (I - mu)^2 - SIc^2
 };
 
-// Per-block scratch of the half-sweep's pooled candidate evaluation: each
-// pixel's reference statistics and the minimum (cost, candidate) key of its
-// neighbour candidates, and per warp the list of (lane, candidate) pairs that
+// Per-block scratch of the half-sweep's pooled candidate evaluation, for a block
+// of N pixels: each pixel's reference statistics and the minimum (cost, candidate) key of its
+// neighbour candidates, and per warp the list of (pixel, candidate) pairs that
 // need a cost evaluation.
+template <int N>
 struct SweepPool {
-    unsigned long long key[BLOCK_THREADS];
-    RefStats st[BLOCK_THREADS];
-    unsigned char item[BLOCK_THREADS / 32][32 * 8];
+    unsigned long long key[N];
+    RefStats st[N];
+    unsigned char item[BLOCK_THREADS / 32][N * 8 / (BLOCK_THREADS / 32)];
 };
 struct NoPool {};
 
@@ -126,7 +127,7 @@ struct BoundPool {
 // one colour and TPP threads per pixel, 128 threads in all.
 template <int TW, int TH, int TPP = 1, int HALO = MAX_HALO, bool POOL = TPP == 1, bool BOUND = false>
 struct TileSmemT {
-    static constexpr int W = TW, H = TH;
+    static constexpr int W = TW, H = TH, LANES = TPP;
     static constexpr int PITCH = TW + 2 * HALO, ROWS = TH + 2 * HALO;
     static constexpr int THREADS = (TW / 2) * TH;
     static_assert(THREADS * TPP == BLOCK_THREADS, "every tile shape runs 128 threads");
@@ -136,7 +137,7 @@ struct TileSmemT {
     float col_sin[PITCH], col_cos[PITCH];  // sin lon, cos lon
     float wsp[2 * HALO + 1];             // spatial log2-weight of offset index k
     // candidate pooling of the one-thread-per-pixel half-sweep
-    typename std::conditional<POOL, SweepPool, NoPool>::type pool;
+    typename std::conditional<POOL, SweepPool<THREADS>, NoPool>::type pool;
     // the bounded half-sweep's (36 samples at 11x11 / 2, (2 HALO + 1)^2 at most)
     static constexpr int SAMPLES = HALO == 5 ? 36 : (2 * HALO + 1) * (2 * HALO + 1);
     typename std::conditional<BOUND, BoundPool<TW, TH, HALO, SAMPLES>, NoPool>::type bound;
@@ -147,6 +148,10 @@ using TileSmem = TileSmemT<TILE_W, TILE_H>;  // the batched and no-alloc kernels
 template <int TS, int HALO = MAX_HALO, bool POOL = true> struct TileShape { using Smem = TileSmemT<32, 8, 1, HALO, POOL>; };
 template <int HALO, bool POOL> struct TileShape<1, HALO, POOL> { using Smem = TileSmemT<64, 4, 1, HALO, POOL>; };
 template <int HALO, bool POOL> struct TileShape<2, HALO, POOL> { using Smem = TileSmemT<16, 16, 1, HALO, POOL>; };
+// 2, 4 and 8 lanes per pixel, for keyframes of few tiles (sweep_shape).
+template <int HALO, bool POOL> struct TileShape<3, HALO, POOL> { using Smem = TileSmemT<32, 4, 2, HALO, POOL>; };
+template <int HALO, bool POOL> struct TileShape<4, HALO, POOL> { using Smem = TileSmemT<16, 4, 4, HALO, POOL>; };
+template <int HALO, bool POOL> struct TileShape<5, HALO, POOL> { using Smem = TileSmemT<8, 4, 8, HALO, POOL>; };
 
 // Rotated column directions of the paired path: for view pair q and tile
 // column c, colU[q][k][c] = row k of R_s applied to (sin lon_c, 0, cos lon_c)
@@ -850,11 +855,20 @@ __device__ __forceinline__ void count_close(const PixelParams& P, bool close) {
 // and every pixel keeps the minimum of (cost, candidate index) in shared
 // memory; then each pixel adopts that candidate if it wins and runs its
 // refinements. The maps equal those of trying all candidates in turn.
+//
+// LANES lanes of a warp share a pixel. One (the shape of large keyframes) leaves
+// nothing idle. Several spread a small keyframe over more warps: its neighbour
+// candidates are pooled as ever, and its next LANES refinement tests are scored
+// side by side from the same incumbent, on the supposition that all but the last
+// fail; the first success is taken, and the tests after it are scored again from
+// the new incumbent. The maps are those of the tests in turn.
 template <int NS, bool EXACT, class VA, int WIN, class SM>
-__device__ __forceinline__ void sweep_pooled(const PixelParams& P, SM& sm, int bx, int by, int x, int y, int colour,
-                                             int iter) {
-    const bool active = x < P.W && y < P.H;
+__device__ __forceinline__ void sweep_pooled(const PixelParams& P, SM& sm, int bx, int by, int colour, int iter) {
+    constexpr int LANES = SM::LANES, PER_WARP = 32 / LANES;
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    const int sub = lane % LANES, own = threadIdx.x / LANES;  // this lane of its pixel's; its pixel of the block
+    const int y = by + own / (SM::W / 2), x = bx + 2 * (own % (SM::W / 2)) + ((y + colour) & 1);
+    const bool active = x < P.W && y < P.H;
     const int lx = x - bx + P.radius, ly = y - by + P.radius;
     const size_t i = (size_t)y * P.W + x;
     float bd = 0.f, bc = 0.f;
@@ -862,17 +876,19 @@ __device__ __forceinline__ void sweep_pooled(const PixelParams& P, SM& sm, int b
     unsigned need = 0;
     bool replaced = false;
     if (active) {
+        rp = make_float3(sm.row_cos[ly] * sm.col_sin[lx], -sm.row_sin[ly], sm.row_cos[ly] * sm.col_cos[lx]);
+        bd = P.depth[i];
+        bn = make_float3(P.nx[i], P.ny[i], P.nz[i]);
+        bc = P.cost[i];
+    }
+    if (active && sub == 0) {
         unsigned settled = 0;  // neighbours whose plane was tried in the last half-sweep
         if (P.changed != nullptr && iter > 0) {
 #pragma unroll
             for (int k = 0; k < 8; ++k) settled |= (unsigned)unchanged_neighbour(P, x, y, k) << k;
         }
-        rp = make_float3(sm.row_cos[ly] * sm.col_sin[lx], -sm.row_sin[ly], sm.row_cos[ly] * sm.col_cos[lx]);
         float SII, w_centre;
-        sm.pool.st[threadIdx.x] = ref_stats<WIN>(P, sm, lx, ly, SII, w_centre);
-        bd = P.depth[i];
-        bn = make_float3(P.nx[i], P.ny[i], P.nz[i]);
-        bc = P.cost[i];
+        sm.pool.st[own] = ref_stats<WIN>(P, sm, lx, ly, SII, w_centre);
         float cd[8];
         float3 cn[8];
 #pragma unroll
@@ -884,7 +900,7 @@ __device__ __forceinline__ void sweep_pooled(const PixelParams& P, SM& sm, int b
             if (ok && !dup && !((settled >> k) & 1u)) need |= 1u << k;
         }
     }
-    sm.pool.key[threadIdx.x] = ~0ull;
+    if (sub == 0) sm.pool.key[own] = ~0ull;
     // this lane's first slot in the warp's list: exclusive prefix of the counts
     const int cnt = __popc(need);
     int off = cnt;
@@ -896,16 +912,15 @@ __device__ __forceinline__ void sweep_pooled(const PixelParams& P, SM& sm, int b
     const int total = __shfl_sync(0xffffffffu, off, 31);
     off -= cnt;
     unsigned char* items = sm.pool.item[warp];
-    for (unsigned m = need; m; m &= m - 1) items[off++] = (unsigned char)((lane << 3) | (__ffs(m) - 1));
+    for (unsigned m = need; m; m &= m - 1) items[off++] = (unsigned char)(((lane / LANES) << 3) | (__ffs(m) - 1));
     __syncwarp();
 
     const int pooled_rounds = (total + 31) >> 5;  // warp-uniform
-    const int n_jobs = pooled_rounds + P.n_refine;
     const float span = P.inv_dmin - P.inv_dmax;
     // the neighbour phase's winner, once every pooled evaluation has landed
     auto adopt_best = [&]() {
         __syncwarp();
-        const unsigned long long key = sm.pool.key[threadIdx.x];
+        const unsigned long long key = sm.pool.key[own];
         if (active && key != ~0ull) {
             const float c = from_ordered_bits((unsigned)(key >> 3));
             if (c < bc) {
@@ -919,12 +934,17 @@ __device__ __forceinline__ void sweep_pooled(const PixelParams& P, SM& sm, int b
             }
         }
     };
+    int taken = 0;  // refinement tests of the own pixel decided (one lane a pixel: the same in all)
 #pragma unroll 1
-    for (int r = 0; r < n_jobs; ++r) {
-        if (r == pooled_rounds) adopt_best();
+    for (int r = 0;; ++r) {
+        if (r >= pooled_rounds) {
+            if (r == pooled_rounds) adopt_best();
+            if (LANES == 1 ? r == pooled_rounds + P.n_refine : !__any_sync(0xffffffffu, active && taken < P.n_refine)) break;
+            if (LANES == 1) taken = r - pooled_rounds;
+        }
         // the job of this round: (pixel, plane)
         bool job = false;
-        int jt = threadIdx.x, jx = x, jy = y, k = 0;
+        int jt = own, jx = x, jy = y, k = 0;
         float3 jrp = rp;
         float dc = 0.f;
         float3 nc = make_float3(0.f, 0.f, 0.f);
@@ -933,14 +953,14 @@ __device__ __forceinline__ void sweep_pooled(const PixelParams& P, SM& sm, int b
             if (idx < total) {
                 const int it = items[idx];
                 k = it & 7;
-                jt = (warp << 5) + (it >> 3);
+                jt = warp * PER_WARP + (it >> 3);
                 const int otx = jt % (SM::W / 2), oty = jt / (SM::W / 2);
                 jy = by + oty;
                 jx = bx + 2 * otx + ((jy + colour) & 1);
                 job = true;
             }
-        } else if (active) {
-            const int t = r - pooled_rounds;
+        } else if (active && taken + sub < P.n_refine) {
+            const int t = taken + sub;
             const float sc = __int_as_float((126 - t) << 23);  // 2^-(t+1)
             const U4 u = draw_uniform4(i, (uint64_t)iter, (uint64_t)(1 + t), P.seed, P.keyframe);
             float inv = fmaf((2.0f * u.x - 1.0f) * sc, span, 1.0f / bd);
@@ -952,26 +972,48 @@ __device__ __forceinline__ void sweep_pooled(const PixelParams& P, SM& sm, int b
             nc = face_camera(make_float3(nc.x * il, nc.y * il, nc.z * il), rp);
             job = true;
         }
-        if (!job) continue;
-        const int jlx = jx - bx + P.radius, jly = jy - by + P.radius;
-        if (r < pooled_rounds) {
-            jrp = make_float3(sm.row_cos[jly] * sm.col_sin[jlx], -sm.row_sin[jly], sm.row_cos[jly] * sm.col_cos[jlx]);
-            neighbour_candidate(P, jx, jy, jrp, k, dc, nc);
+        if (LANES == 1 && !job) continue;
+        float c = 4.0f;  // above every cost
+        bool won = false;
+        if (job) {
+            const int jlx = jx - bx + P.radius, jly = jy - by + P.radius;
+            if (r < pooled_rounds) {
+                jrp = make_float3(sm.row_cos[jly] * sm.col_sin[jlx], -sm.row_sin[jly], sm.row_cos[jly] * sm.col_cos[jlx]);
+                neighbour_candidate(P, jx, jy, jrp, k, dc, nc);
+            }
+            c = cost_of<NS, EXACT, VA, WIN, SM, true>(P, sm, jlx, jly, sm.pool.st[jt], jrp, dc, nc);
+            if (r < pooled_rounds) {
+                if (c == c) atomicMin(&sm.pool.key[jt], ((unsigned long long)ordered_bits(c) << 3) | (unsigned)k);
+            } else {
+                won = c < bc;
+            }
         }
-        const float c = cost_of<NS, EXACT, VA, WIN, SM, true>(P, sm, jlx, jly, sm.pool.st[jt], jrp, dc, nc);
-        if (r < pooled_rounds) {
-            if (c == c) atomicMin(&sm.pool.key[jt], ((unsigned long long)ordered_bits(c) << 3) | (unsigned)k);
-        } else if (c < bc) {
-            bc = c;
-            bd = dc;
-            bn = nc;
-            replaced = true;
+        if constexpr (LANES == 1) {
+            if (won) {
+                bc = c;
+                bd = dc;
+                bn = nc;
+                replaced = true;
+            }
+        } else if (r >= pooled_rounds) {
+            // the pixel's first success, if there is one, becomes every lane's incumbent
+            const unsigned mine = (__ballot_sync(0xffffffffu, won) >> (lane - sub)) & ((1u << LANES) - 1u);
+            const int first = mine ? __ffs(mine) - 1 : sub, from = lane - sub + first;
+            const float cw = __shfl_sync(0xffffffffu, c, from), dw = __shfl_sync(0xffffffffu, dc, from);
+            const float3 nw = make_float3(__shfl_sync(0xffffffffu, nc.x, from), __shfl_sync(0xffffffffu, nc.y, from),
+                                          __shfl_sync(0xffffffffu, nc.z, from));
+            if (mine) {
+                bc = cw;
+                bd = dw;
+                bn = nw;
+                replaced = true;
+            }
+            taken += mine ? first + 1 : LANES;
         }
     }
-    if (n_jobs == pooled_rounds) adopt_best();
-    if constexpr (has_bounded(NS, EXACT) && std::is_same<VA, ParamViews>::value)
+    if constexpr (has_bounded(NS, EXACT) && std::is_same<VA, ParamViews>::value && LANES == 1)
         if (P.close != nullptr) count_close(P, active && bc < CLOSE_COST);
-    if (!active) return;
+    if (!active || sub != 0) return;
     if (P.changed) P.changed[i] = replaced;
     P.depth[i] = bd;
     P.nx[i] = bn.x;
@@ -1530,9 +1572,7 @@ __device__ __forceinline__ void process_tile(const PixelParams& P, SM& sm, int b
                                              int iter) {
     prepare_tile<NS, EXACT, VA>(P, sm, bx, by);
     if constexpr (MODE == MODE_SWEEP) {
-        const int y = by + threadIdx.x / (SM::W / 2);
-        const int x = bx + 2 * (threadIdx.x % (SM::W / 2)) + ((y + colour) & 1);
-        sweep_pooled<NS, EXACT, VA, WIN, SM>(P, sm, bx, by, x, y, colour, iter);
+        sweep_pooled<NS, EXACT, VA, WIN, SM>(P, sm, bx, by, colour, iter);
     } else {
         score_pixel<NS, EXACT, MODE, VA, WIN>(P, sm, bx, by, colour);
     }
@@ -1621,7 +1661,7 @@ template <int NS, bool EXACT, int MODE, int WIN>
 inline void launch_score(const PixelParams& p, cudaStream_t stream) {
     prefer_texture_cache<pixel_kernel<NS, EXACT, MODE, WIN, 0>>();
     dim3 grid = tile_grid<0>(p);
-    grid.z = (long long)grid.x * grid.y >= 8 * 152 ? 1 : 2;
+    grid.z = (long long)grid.x * grid.y >= 8 * SM_COUNT ? 1 : 2;
     pixel_kernel<NS, EXACT, MODE, WIN, 0><<<grid, BLOCK_THREADS, 0, stream>>>(p);
 }
 template <int NS, bool EXACT, int MODE>
@@ -1644,12 +1684,30 @@ inline void launch_bounded(const PixelParams& p, cudaStream_t stream) {
     }
 }
 
-// A fixed-window sweep in the problem's tile shape.
+// The tile shape of a half-sweep: the one asked for, else 32x8 with as many lanes
+// per pixel as its tiles, with those of the keyframes beside it, leave room for
+// (tiles x lanes within 5/6 of the resident blocks). Whole runs, ms at 1, 2, 4 and 8
+// lanes: 64x32 of 2 views (8 tiles) 1.59 1.08 0.83 0.72; 256x128 (128 tiles) of 2 views
+// 1.66 1.22 1.18 1.39, of 6 views 3.47 2.83 3.12 3.59; 320x160 of 4 (200) 2.02 1.66 1.94
+// 2.13; 384x192 (288) of 2 views 1.91 1.69 2.10 2.42, of 6 views 4.55 4.62 5.51 6.66;
+// 512x256 of 2 (512) 2.63 2.81 3.19 3.96.
+template <int NS>
+inline int sweep_shape(const PixelParams& p) {
+    if (p.tile != 0) return p.tile;
+    const long long tiles = (long long)((p.W + TILE_W - 1) / TILE_W) * ((p.H + TILE_H - 1) / TILE_H) + p.crowd;
+    const long long resident = (long long)SM_COUNT * pixel_min_blocks(NS);
+    return 8 * tiles * 6 <= resident * 5 ? 5 : 4 * tiles * 6 <= resident * 5 ? 4 : 2 * tiles * 6 <= resident * 5 ? 3 : 0;
+}
+
+// A sweep in its tile shape.
 template <int NS, bool EXACT, int WIN>
 inline void launch_sweep_window(const PixelParams& p, cudaStream_t stream) {
-    switch (p.tile) {
-        case 1: launch_tiles<NS, EXACT, MODE_SWEEP, WIN, 1>(p, stream); break;
-        case 2: launch_tiles<NS, EXACT, MODE_SWEEP, WIN, 2>(p, stream); break;
+    switch (sweep_shape<NS>(p)) {
+        case 1: launch_tiles<NS, EXACT, MODE_SWEEP, WIN, WIN ? 1 : 0>(p, stream); break;
+        case 2: launch_tiles<NS, EXACT, MODE_SWEEP, WIN, WIN ? 2 : 0>(p, stream); break;
+        case 3: launch_tiles<NS, EXACT, MODE_SWEEP, WIN, 3>(p, stream); break;
+        case 4: launch_tiles<NS, EXACT, MODE_SWEEP, WIN, 4>(p, stream); break;
+        case 5: launch_tiles<NS, EXACT, MODE_SWEEP, WIN, 5>(p, stream); break;
         default: launch_tiles<NS, EXACT, MODE_SWEEP, WIN, 0>(p, stream); launch_bounded<NS, EXACT, WIN>(p, stream); break;
     }
 }
@@ -1686,8 +1744,7 @@ cudaError_t launch_pixel_kernel_ns(const PixelParams& p, int mode, cudaStream_t 
                     break;
                 }
             }
-            launch_tiles<NS, EXACT, MODE_SWEEP>(p, stream);
-            launch_bounded<NS, EXACT, 0>(p, stream);
+            launch_sweep_window<NS, EXACT, 0>(p, stream);
             break;
     }
     return cudaGetLastError();

@@ -171,12 +171,8 @@ cudaError_t bind_history(PixelParams& P, uint8_t* mem, int iterations, cudaStrea
     P.changed = mem;
     P.close = nullptr;
     if (!mem || P.S < 4 || P.S > 10 || P.tile != 0 || P.tpp > 1 || P.tpp < -1) return cudaSuccess;
-    int dev = 0, sms = 0;
-    cudaError_t e = cudaGetDevice(&dev);
-    if (e == cudaSuccess) e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
-    if (e != cudaSuccess) return e;
     const long long tiles = (long long)((P.W + TILE_W - 1) / TILE_W) * ((P.H + TILE_H - 1) / TILE_H);
-    if (tiles < 3ll * sms) return cudaSuccess;
+    if (tiles < 3ll * SM_COUNT) return cudaSuccess;
     P.close = reinterpret_cast<unsigned*>(mem + (((size_t)P.W * P.H + 255) & ~size_t(255)));
     return cudaMemsetAsync(P.close, 0, 2 * sizeof(unsigned) * (size_t)iterations, st);
 }

@@ -245,6 +245,7 @@ int enqueue_tail(Serving& s, Request* r, cudaStream_t st) {
 // half-sweeps, then the tail.
 int enqueue_request(Serving& s, Request* r, cudaStream_t st) {
     PixelParams P = r->prob;
+    P.crowd = (int)std::min<size_t>(s.running_tiles, 1 << 24);
     cudaError_t e = cudaSuccess;
     if (history_bytes(r->W, r->H, r->params.iterations) <= (size_t)r->W * r->H * sizeof(float))
         e = bind_history(P, P.changed, r->params.iterations, st);

@@ -60,6 +60,31 @@ def _same(a, b):
     return all(np.array_equal(x, y) for x, y in zip(a, b))
 
 
+# one, two, four and eight lanes a pixel (by size and view count): the same maps with one, in the shapes and the
+# company that get one, and in the persistent kernel
+LANE_FORMS = [(64, 32, 2, "u8", 7, 1, 0, 1, 6), (8, 4, 1, "f32", 5, 1, 0, 1, 5), (130, 66, 6, "f16", 11, 2, 1, 3, 7),
+              (256, 128, 2, "u8", 7, 1, 0, 1, 6), (250, 130, 3, "f32", 9, 3, 1, 2, 13), (256, 130, 6, "u8", 11, 2, 0, 3, 6),
+              (322, 158, 4, "f16", 11, 2, 0, 4, 1), (384, 194, 2, "u8", 13, 2, 0, 2, 0), (66, 34, 16, "u8", 5, 1, 0, 7, 6)]
+
+
+@pytest.mark.parametrize("form", LANE_FORMS)
+def test_lanes_per_pixel_change_nothing(pm, form):
+    prob, params = _problem(form, 4)
+    with pm.Context(0) as ctx:
+        want = _steps(pm, ctx, prob, params)
+        assert _same(_bits(pm, ctx, pm.pmsp_densify(ctx, *prob, params)), want)
+        # a tile shape asked for is served by one lane a pixel (11x11 / 2 and 7x7 windows), and so is a keyframe in a crowd
+        for tile, n in ((1, 1), (0, 1 if form[0] > 300 else 60)):
+            batch = pm.Batch([(*prob, params, None)] * n)
+            pm.pmsp_densify_batch(ctx, batch, 0, pm.pmsp_tuning(0, 0, 0, 1, tile, 1, 0))
+            for out in batch.outs[::max(1, n // 3)]:
+                assert _same(_bits(pm, ctx, out), want)
+        batch = pm.Batch([(*prob, params, None)])
+        pm.pmsp_densify_batch(ctx, batch, 0, pm.pmsp_tuning(0, 0, 0, 0, 0, 1, 0))
+        if form[2] <= 10:  # (above, the persistent kernel scores view by view)
+            assert _same(_bits(pm, ctx, batch.outs[0]), want)
+
+
 @pytest.mark.parametrize("form", FORMS)
 def test_run_equals_its_steps(pm, form):
     import torch
