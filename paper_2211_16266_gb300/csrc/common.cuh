@@ -91,6 +91,7 @@ struct FilterView {
     int W, H;
     float Rf[9], tf[3];  // reference -> neighbour
     float Rb[9], tb[3];  // neighbour -> reference
+    float su, ou, sv, ov;  // its projection scales, set by launch_filter_kernel
 };
 
 struct FilterParams {
@@ -100,6 +101,7 @@ struct FilterParams {
     int32_t* agree;
     int W, H, n, min_views;
     float max_px;
+    float wrap_hi, wrap_lo, max_sq;  // set by launch_filter_kernel
 };
 
 // Plane-map warping from the previous keyframe into the current one.

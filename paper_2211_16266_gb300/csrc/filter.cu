@@ -13,11 +13,13 @@
 // and neighbour, against 4 bytes read. The bearing needs sines and cosines of the
 // neighbour pixel's row and column only, so each block tabulates them once, for
 // every panorama size among the maps (usually one: 23 KB at 1920x960), and walks
-// the image with a fixed grid (266 instructions per pixel and neighbour are left,
-// issued in 78 % of the slots). 1920x960 against 4 maps: 78.7 -> 73.3 us, against
-// 7.6 us for its 52 MB.
+// the image with a fixed grid. 1920x960 against 4 maps: 79.7 -> 69.8 us a call with
+// the tables, 64.9 with the wrap and the distance as comparisons, against 7.6 us for
+// its 52 MB.
 #include <algorithm>
 #include <atomic>
+#include <cmath>
+#include <limits>
 
 #include "camera.cuh"
 #include "common.cuh"
@@ -84,8 +86,7 @@ __global__ void __launch_bounds__(FILTER_THREADS, FILTER_BLOCKS)
                 const FilterView& V = P.nb[j];
                 const float3 Y = apply(V.Rf, V.tf, X);
                 float uc, vc;
-                project_dir_fast(Y.x, Y.y, Y.z, V.W * 0.15915494309189535f, 0.5f * V.W - 0.5f,
-                            -V.H * 0.3183098861837907f, 0.5f * V.H - 0.5f, uc, vc);
+                project_dir_fast(Y.x, Y.y, Y.z, V.su, V.ou, V.sv, V.ov, uc, vc);
                 // |lon| <= pi: the rounded column lies within one of [0, W)
                 int ui = (int)floorf(uc + 0.5f);
                 ui = ui < 0 ? ui + V.W : (ui >= V.W ? ui - V.W : ui);
@@ -98,9 +99,9 @@ __global__ void __launch_bounds__(FILTER_THREADS, FILTER_BLOCKS)
                 float u2, v2;
                 project_dir_fast(Z.x, Z.y, Z.z, su, ou, sv, ov, u2, v2);
                 float du = u2 - (float)x;
-                du -= P.W * floorf(du / P.W + 0.5f);
+                du = du >= P.wrap_hi ? du - P.W : (du < P.wrap_lo ? du + P.W : du);  // into half a panorama
                 const float dv = v2 - (float)y;
-                if (sqrtf(du * du + dv * dv) < P.max_px) ++cnt;
+                if (du * du + dv * dv < P.max_sq) ++cnt;  // the distance is below max_px
             }
         }
         P.depth_out[i] = (d > 0.f && cnt >= P.min_views) ? d : 0.f;
@@ -108,7 +109,37 @@ __global__ void __launch_bounds__(FILTER_THREADS, FILTER_BLOCKS)
     }
 }
 
-cudaError_t launch_filter_kernel(const FilterParams& p, cudaStream_t stream) {
+// The smallest float x for which `pred` holds, pred being monotone (false, then
+// true), from a guess a few floats away.
+template <class Pred>
+static float first_float(float x, Pred pred) {
+    const float inf = std::numeric_limits<float>::infinity();
+    while (!pred(x) && x < inf) x = std::nextafter(x, inf);
+    for (float below = std::nextafter(x, -inf); pred(below); below = std::nextafter(x, -inf)) x = below;
+    return x;
+}
+
+cudaError_t launch_filter_kernel(const FilterParams& params, cudaStream_t stream) {
+    FilterParams p = params;
+    // The wrap of a longitude difference du by whole panoramas, du - W floor(du / W + 1/2),
+    // and sqrt(s) < max_px as comparisons with the floats at which their FP32 values turn
+    // (|du| < W: the floor is -1, 0 or 1), so that the kernel neither divides nor takes roots.
+    const float W = (float)p.W;
+    auto turns = [&](float du) {
+        volatile float q = du / W;
+        volatile float h = q + 0.5f;
+        return std::floor(h);
+    };
+    p.wrap_hi = first_float(0.5f * W, [&](float du) { return turns(du) >= 1.0f; });
+    p.wrap_lo = first_float(-0.5f * W, [&](float du) { return turns(du) >= 0.0f; });
+    p.max_sq = first_float(p.max_px * p.max_px, [&](float s) { return s > 0.0f && std::sqrt(s) >= p.max_px; });
+    for (int j = 0; j < p.n; ++j) {
+        FilterView& V = p.nb[j];
+        V.su = V.W * 0.15915494309189535f;
+        V.ou = 0.5f * V.W - 0.5f;
+        V.sv = -V.H * 0.3183098861837907f;
+        V.ov = 0.5f * V.H - 0.5f;
+    }
     FilterTables T{};
     size_t entries = 0;
     auto table_of = [&](int W, int H) {
