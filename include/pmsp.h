@@ -294,8 +294,9 @@ int pmsp_view_filter(pmsp_ctx* ctx, const pmsp_pose* a, const pmsp_pose* b, cons
  *   count    host int64 receiving the number of occupied voxels (call with
  *            cap = 0 to size the output)
  * Synchronous. Device memory, held by the context between calls: a hash table
- * of 16 bytes per slot (a power of two >= a quarter of the input pixels; where
- * the voxels do not fit, up to one >= twice the pixels) and a bit per pixel. Errors: PMSP_EINVAL for NULL or mismatched
+ * of 16 bytes per slot (a power of two >= twice the input pixels up to 2^22,
+ * then one >= a quarter of them; where the voxels do not fit, up to one >= twice
+ * the pixels) and a bit per pixel. Errors: PMSP_EINVAL for NULL or mismatched
  * arguments, voxel <= 0, or a point beyond the key range.
  */
 int pmsp_fuse(pmsp_ctx* ctx, const pmsp_maps* maps, const pmsp_pose* poses, int n, float voxel, float* points,

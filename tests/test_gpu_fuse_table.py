@@ -21,8 +21,9 @@ def _first_of_voxels(points, voxel):
 
 
 @pytest.mark.parametrize("sizes,voxel", [
-    ([(64, 32)], 1e-3),                    # every pixel a voxel of its own: the table grows to its largest
-    ([(640, 320), (333, 167)], 2e-3),      # grows once
+    ([(64, 32)], 1e-3),                    # every pixel a voxel of its own
+    ([(640, 320), (333, 167)], 2e-3),
+    ([(2048, 1024), (2048, 1024)], 1e-3),  # more voxels than a table within L2 takes: it grows
     ([(33, 9), (32, 8), (31, 7)], 0.05),   # edges of the 32 x 8 tiles
     ([(1, 1)], 0.02), ([(257, 1), (1, 65)], 0.2),
     ([(320, 160)] * 16, 0.5),              # many pixels to a voxel, the most keyframes
