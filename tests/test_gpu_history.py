@@ -29,7 +29,7 @@ FORMS = [  # W, H, views, format, window, stride, table, best_k, n_refine
     # from 456 tiles on: the refinement tests dropped by a bound, in every window class, ragged, with more tests
     # than are drawn ahead, with none, with no bilateral weights and with the mean over all views
     (518, 250, 4, "u8", 11, 2, 0, 1, 6), (512, 256, 5, "f16", 7, 1, 1, 5, 9), (640, 200, 6, "f32", 9, 3, 0, 3, 6),
-    (514, 258, 7, "u8", 11, 2, 1, 2, 0), (512, 260, 10, "u8", 11, 2, 0, 3, 30),
+    (512, 258, 6, "f32", 9, 2, 0, 3, 6), (514, 258, 7, "u8", 11, 2, 1, 2, 0), (512, 260, 10, "u8", 11, 2, 0, 3, 30),
 ]
 
 
