@@ -17,7 +17,6 @@
 // the tables, 64.9 with the wrap and the distance as comparisons, against 7.6 us for
 // its 52 MB.
 #include <algorithm>
-#include <atomic>
 #include <cmath>
 #include <limits>
 
@@ -164,12 +163,8 @@ cudaError_t launch_filter_kernel(const FilterParams& params, cudaStream_t stream
     const long long resident = (long long)FILTER_BLOCKS * sms, per_block = (long long)p.W * p.H * p.n / std::min(resident, work);
     if (bytes <= FILTER_TABLE_BYTES && per_block >= 2ll * (long long)entries) {
         if (bytes > 48 * 1024) {
-            static std::atomic<uint64_t> allowed{0};
-            if (dev >= 64 || !((allowed.load(std::memory_order_relaxed) >> dev) & 1)) {
-                e = cudaFuncSetAttribute(filter_kernel<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, FILTER_TABLE_BYTES);
-                if (e != cudaSuccess) return e;
-                if (dev < 64) allowed.fetch_or(1ull << dev, std::memory_order_relaxed);
-            }
+            e = cudaFuncSetAttribute(filter_kernel<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, FILTER_TABLE_BYTES);
+            if (e != cudaSuccess) return e;
         }
         filter_kernel<true><<<(unsigned)std::min(resident, work), FILTER_THREADS, bytes, stream>>>(p, T);
     } else {
