@@ -267,7 +267,9 @@ def run_gpu(args):
                                units_basis="the method's 8 neighbour + 6 refinement candidates per pixel, 6 views, "
                                            "36 samples; the kernel skips neighbour candidates bit-identical to the "
                                            "incumbent or an earlier one (about 4.4 % of the evaluation rounds on "
-                                           "this workload), whose cost is known",
+                                           "this workload), whose cost is known; timed as half-sweeps called on their own, "
+                                           "while those of a run also leave out neighbours they know and refinement "
+                                           "tests that cannot win",
                                units=dict(
                                    # one gather and four special-function results per view-sample
                                    gather_frac_of_l1_peak=achieved / peaks["gather_l1_per_s"],
