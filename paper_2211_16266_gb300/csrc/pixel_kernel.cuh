@@ -935,13 +935,17 @@ __device__ __forceinline__ void sweep_pooled(const PixelParams& P, SM& sm, int b
         }
     };
     int taken = 0;  // refinement tests of the own pixel decided (one lane a pixel: the same in all)
+    // With one lane a pixel the bound of the loop is known: leaving it by the test of
+    // several lanes took 2.60 ms where this takes 2.52 (1000x502, 4 views, 9x9 at stride
+    // 3, 3 iterations) and 10.07 where this takes 9.76 (8 views, 5x5).
+    const int n_jobs = pooled_rounds + P.n_refine;
 #pragma unroll 1
-    for (int r = 0;; ++r) {
-        if (r >= pooled_rounds) {
-            if (r == pooled_rounds) adopt_best();
-            if (LANES == 1 ? r == pooled_rounds + P.n_refine : !__any_sync(0xffffffffu, active && taken < P.n_refine)) break;
-            if (LANES == 1) taken = r - pooled_rounds;
-        }
+    for (int r = 0; LANES != 1 || r < n_jobs; ++r) {
+        if (r == pooled_rounds) adopt_best();
+        if (LANES == 1)
+            taken = r - pooled_rounds;
+        else if (r >= pooled_rounds && !__any_sync(0xffffffffu, active && taken < P.n_refine))
+            break;
         // the job of this round: (pixel, plane)
         bool job = false;
         int jt = own, jx = x, jy = y, k = 0;
@@ -1011,6 +1015,7 @@ __device__ __forceinline__ void sweep_pooled(const PixelParams& P, SM& sm, int b
             taken += mine ? first + 1 : LANES;
         }
     }
+    if (LANES == 1 && n_jobs == pooled_rounds) adopt_best();
     if constexpr (has_bounded(NS, EXACT) && std::is_same<VA, ParamViews>::value && LANES == 1)
         if (P.close != nullptr) count_close(P, active && bc < CLOSE_COST);
     if (!active || sub != 0) return;
