@@ -391,7 +391,8 @@ typedef struct {
                               1: every keyframe's own launch chain, chains run concurrently on
                                  parallel streams (parallel branches of the captured graph) */
     int32_t tile;          /* strategy 1, half-sweeps with an 11x11/2 or 7x7/1 window: tile of
-                              reference pixels per 128-thread block, 0: 32x8, 1: 64x4, 2: 16x16
+                              reference pixels per 128-thread block, 0: 32x8 (smaller with
+                              several threads per pixel where tiles are few), 1: 64x4, 2: 16x16
                               (every shape computes the same numbers) */
     int32_t tpp;           /* strategy 1, half-sweeps of keyframes with 2 or more sources:
                               threads per pixel, 0 or 1: one; 2, 4 (or 8 with `lanes` 1):
