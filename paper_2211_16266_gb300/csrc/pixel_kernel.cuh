@@ -33,6 +33,7 @@
 #include "camera.cuh"
 #include "common.cuh"
 #include "philox.cuh"
+#include "sweep_policy.h"
 
 namespace pmsp {
 
@@ -818,16 +819,12 @@ __device__ __forceinline__ float from_ordered_bits(unsigned o) {
 // View counts with a bounded half-sweep (launch_pixel_kernel_ns).
 constexpr bool has_bounded(int ns, bool exact) { return exact && ns >= 4 && ns <= 10; }
 
-// Pixels whose incumbent costs less than this: enough of a refinement test's samples
-// bound its cost above them.
-constexpr float CLOSE_COST = 0.15f;
-
-// Whether the half-sweep of (iter, colour) goes to the bounded kernel: half of the
-// pixels of the half-sweep before it ended close. Every half-sweep of such a run
+// Whether the half-sweep of (iter, colour) goes to the bounded kernel: enough of the
+// pixels of the half-sweep before it ended close (sweep_policy.h). Every half-sweep of such a run
 // is launched as both kernels, and one of them finds that it is not its turn.
 __device__ __forceinline__ bool bounded_turn(const PixelParams& P) {
     const int phase = 2 * P.iter + P.colour;
-    return phase > 0 && P.close[phase - 1] >= (unsigned)((long long)P.W * P.H / 4);
+    return phase > 0 && P.close[phase - 1] >= (unsigned)bounded_from(P.W, P.H);
 }
 
 // The half-sweep's close pixels, for the next one's choice (the block calls it).

@@ -14,6 +14,7 @@
 #include "common.cuh"
 #include "pmsp.h"
 #include "runtime.h"
+#include "sweep_policy.h"
 
 using namespace pmsp;
 
@@ -163,18 +164,12 @@ size_t history_bytes(int W, int H, int iterations) {
 
 // Gives P its history in `mem` (history_bytes; may be NULL), the counters zeroed in
 // the order of `st`. The counters let half-sweeps go to the bounded kernel where it
-// pays: its views (4 to 10: 1920x960, 8 iterations, 3 views of 7x7 35.3 against 35.1
-// ms), a window with samples left to drop (5 x 5 or more: 1414x706, 6 views, 3 iterations
-// with noise, 9x9 at stride 3, 9 samples: 7.02 against 6.30 ms; 8 iterations without
-// noise 14.69 against 14.62, at stride 2, 25 samples, 29.3 against 33.6) and a grid that keeps the GPU busy while lanes of a warp wait for one another
-// (384x192, 288 tiles, 6 views: 4.6 against 4.8 ms pooled; 640x320, 800 tiles: 10.8
-// against 9.8).
+// may serve them (sweep_policy.h).
 cudaError_t bind_history(PixelParams& P, uint8_t* mem, int iterations, cudaStream_t st) {
     P.changed = mem;
     P.close = nullptr;
-    if (!mem || P.S < 4 || P.S > 10 || 2 * P.radius < 4 * P.stride || P.tile != 0 || P.tpp > 1 || P.tpp < -1) return cudaSuccess;
     const long long tiles = (long long)((P.W + TILE_W - 1) / TILE_W) * ((P.H + TILE_H - 1) / TILE_H);
-    if (tiles < 3ll * SM_COUNT) return cudaSuccess;
+    if (!mem || P.tile != 0 || P.tpp > 1 || P.tpp < -1 || !bounded_serves(P.S, P.K, tiles, SM_COUNT)) return cudaSuccess;
     P.close = reinterpret_cast<unsigned*>(mem + (((size_t)P.W * P.H + 255) & ~size_t(255)));
     return cudaMemsetAsync(P.close, 0, 2 * sizeof(unsigned) * (size_t)iterations, st);
 }
