@@ -637,13 +637,22 @@ __device__ __forceinline__ void pairs_sample(const PixelParams& P, float alpha, 
     pairs_sample_columns<NP, VA>(P, alpha, beta, U, J);
 }
 
+// Half-sweeps that read the column table by shared addresses: those of even view
+// counts (1920x960, 6 views, 8 iterations: 76.8 -> 75.8 ms; 3840x1920, 8 views: 390 ->
+// 380 ms), but only the fixed windows with 6 views, and with 8 where a lane has a pixel of its
+// own (one iteration at 13x13 / 2, by address and by index: 514x258, 6 views 1736 against
+// 1709 us, 1000x502 5493 against 5434, 8 views 7022 against 6998; 4 iterations of 9x9 / 2, 8
+// views, lanes a pixel: 256x128 1631 against 1687; 1920x960, 13x13 / 2, 10 views 30472 against
+// 30636, 2 views 7728 against 8106). With an odd last view, and in the one-evaluation
+// kernels, indexing is the faster (5 views 8.83 against 8.91 ms, the cost of 6 views 1.03
+// against 1.05 ms).
+constexpr bool columns_at_address(int ns, int win, int lanes) {
+    return ns % 2 == 0 && (win != 0 || (ns != 6 && (ns != 8 || lanes > 1)));
+}
+
 // plane_cost for exactly NS >= 2 views held in kernel parameters, with the
 // views processed in pairs (packed FP32) and an odd last view on its own.
-// AT_ADDRESS: the column table by shared addresses, in the half-sweeps of even
-// view counts (1920x960, 6 views, 8 iterations: 76.8 -> 75.8 ms; 3840x1920, 8
-// views: 390 -> 380 ms). With an odd last view, and in the one-evaluation
-// kernels, indexing is the faster (5 views 8.83 against 8.91 ms, the cost of 6
-// views 1.03 against 1.05 ms).
+// AT_ADDRESS: the column table by shared addresses, where columns_at_address says so.
 template <int NS, int WIN, class SM, class VA, bool AT_ADDRESS>
 __device__ __forceinline__ float plane_cost_paired(const PixelParams& P, const SM& sm, int lx, int ly,
                                                    const RefStats& st, float3 rp, float d, float3 n) {
@@ -747,7 +756,7 @@ template <int NS, bool EXACT, class VA, int WIN = 0, class SM = TileSmem, bool S
 __device__ __forceinline__ float cost_of(const PixelParams& P, const SM& sm, int lx, int ly,
                                          const RefStats& st, float3 rp, float d, float3 n) {
     if constexpr (EXACT && NS >= 2 && paired_views<VA>())
-        return plane_cost_paired<NS, WIN, SM, VA, SWEEP && NS % 2 == 0>(P, sm, lx, ly, st, rp, d, n);
+        return plane_cost_paired<NS, WIN, SM, VA, SWEEP && columns_at_address(NS, WIN, SM::LANES)>(P, sm, lx, ly, st, rp, d, n);
     else
         return plane_cost<NS, EXACT, VA, SM>(P, sm, lx, ly, st, rp, d, n);
 }
