@@ -17,11 +17,10 @@
 // the tables, 64.9 with the wrap and the distance as comparisons, against 7.6 us for
 // its 52 MB.
 #include <algorithm>
-#include <cmath>
-#include <limits>
 
 #include "camera.cuh"
 #include "common.cuh"
+#include "filter_thresholds.h"
 
 namespace pmsp {
 
@@ -108,30 +107,12 @@ __global__ void __launch_bounds__(FILTER_THREADS, FILTER_BLOCKS)
     }
 }
 
-// The smallest float x for which `pred` holds, pred being monotone (false, then
-// true), from a guess a few floats away.
-template <class Pred>
-static float first_float(float x, Pred pred) {
-    const float inf = std::numeric_limits<float>::infinity();
-    while (!pred(x) && x < inf) x = std::nextafter(x, inf);
-    for (float below = std::nextafter(x, -inf); pred(below); below = std::nextafter(x, -inf)) x = below;
-    return x;
-}
-
 cudaError_t launch_filter_kernel(const FilterParams& params, cudaStream_t stream) {
     FilterParams p = params;
-    // The wrap of a longitude difference du by whole panoramas, du - W floor(du / W + 1/2),
-    // and sqrt(s) < max_px as comparisons with the floats at which their FP32 values turn
-    // (|du| < W: the floor is -1, 0 or 1), so that the kernel neither divides nor takes roots.
-    const float W = (float)p.W;
-    auto turns = [&](float du) {
-        volatile float q = du / W;
-        volatile float h = q + 0.5f;
-        return std::floor(h);
-    };
-    p.wrap_hi = first_float(0.5f * W, [&](float du) { return turns(du) >= 1.0f; });
-    p.wrap_lo = first_float(-0.5f * W, [&](float du) { return turns(du) >= 0.0f; });
-    p.max_sq = first_float(p.max_px * p.max_px, [&](float s) { return s > 0.0f && std::sqrt(s) >= p.max_px; });
+    const FilterThresholds at = filter_thresholds(p.W, p.max_px);
+    p.wrap_hi = at.wrap_hi;
+    p.wrap_lo = at.wrap_lo;
+    p.max_sq = at.max_sq;
     for (int j = 0; j < p.n; ++j) {
         FilterView& V = p.nb[j];
         V.su = V.W * 0.15915494309189535f;
