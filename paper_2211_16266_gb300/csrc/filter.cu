@@ -13,9 +13,11 @@
 // and neighbour, against 4 bytes read. The bearing needs sines and cosines of the
 // neighbour pixel's row and column only, so each block tabulates them once, for
 // every panorama size among the maps (usually one: 23 KB at 1920x960), and walks
-// the image with a fixed grid. 1920x960 against 4 maps: 79.7 -> 69.8 us a call with
-// the tables, 64.9 with the wrap and the distance as comparisons, against 7.6 us for
-// its 52 MB.
+// the image with a fixed grid, each warp taking 32 pixels of a row at a time. 1920x960
+// against 4 maps, a call alone: 79.7 -> 69.8 us with the tables, 64.9 with the wrap and
+// the distance as comparisons, 61.5 by warps (the rows in strips of 512 left warps idle
+// at most widths), against 7.6 us for its 52 MB. Among other calls: 75.7 -> 57.3 us; 514x257
+// and 8 maps 19.3 -> 11.4.
 #include <algorithm>
 
 #include "camera.cuh"
@@ -30,7 +32,7 @@ __device__ __forceinline__ float3 apply(const float* R, const float* t, float3 X
                        fmaf(R[6], X.x, fmaf(R[7], X.y, fmaf(R[8], X.z, t[2]))));
 }
 
-constexpr int FILTER_THREADS = 512, FILTER_BLOCKS = 3;  // resident blocks per SM
+constexpr int FILTER_WARPS = 16, FILTER_THREADS = 32 * FILTER_WARPS, FILTER_BLOCKS = 3;  // resident blocks per SM
 // Shared memory of the bearing tables in all, for the resident blocks to fit an SM. Maps whose
 // sizes need more get their bearings computed per pixel.
 constexpr size_t FILTER_TABLE_BYTES = 72 * 1024;
@@ -50,7 +52,7 @@ __global__ void __launch_bounds__(FILTER_THREADS, FILTER_BLOCKS)
     extern __shared__ float2 bearings[];
     if constexpr (TABLES) {
         for (int t = 0; t < T.n; ++t)
-            for (int k = threadIdx.x; k < T.H[t] + T.W[t]; k += FILTER_THREADS) {
+            for (int k = threadIdx.x; k < T.H[t] + T.W[t]; k += blockDim.x) {
                 float sn, cs;
                 if (k < T.H[t])
                     sincospif(0.5f - (2.0f * k + 1.0f) / (2.0f * T.H[t]), &sn, &cs);
@@ -68,11 +70,12 @@ __global__ void __launch_bounds__(FILTER_THREADS, FILTER_BLOCKS)
             return pixel_bearing(u, v, W, H);
         }
     };
-    const int strips = (P.W + FILTER_THREADS - 1) / FILTER_THREADS;
+    // a warp takes 32 pixels of a row at a time
+    const int strips = (P.W + 31) / 32, warps = blockDim.x >> 5;
     const float su = P.W * 0.15915494309189535f, ou = 0.5f * P.W - 0.5f;
     const float sv = -P.H * 0.3183098861837907f, ov = 0.5f * P.H - 0.5f;
-    for (int w = blockIdx.x; w < strips * P.H; w += gridDim.x) {
-        const int y = w / strips, x = (w - y * strips) * FILTER_THREADS + threadIdx.x;
+    for (int w = blockIdx.x * warps + (threadIdx.x >> 5); w < strips * P.H; w += gridDim.x * warps) {
+        const int y = w / strips, x = (w - y * strips) * 32 + (threadIdx.x & 31);
         if (x >= P.W) continue;
         const size_t i = (size_t)y * P.W + x;
         const float d = P.depth_in[i];
@@ -138,18 +141,27 @@ cudaError_t launch_filter_kernel(const FilterParams& params, cudaStream_t stream
     cudaError_t e = cudaGetDevice(&dev);
     if (e == cudaSuccess) e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
     if (e != cudaSuccess) return e;
-    const long long work = (long long)((p.W + FILTER_THREADS - 1) / FILTER_THREADS) * p.H;
+    // Strips of 32 pixels, FILTER_WARPS of them at a time in a resident block; where there are
+    // fewer than the resident warps, smaller blocks on more SMs.
+    const long long strips = (long long)((p.W + 31) / 32) * p.H, resident = (long long)FILTER_BLOCKS * sms;
+    const int warps = (int)std::min<long long>(FILTER_WARPS, (strips + resident - 1) / resident);
+    const long long blocks = std::min(resident, (strips + warps - 1) / warps);
     // A block's tables cost as many bearings as the sizes have rows and columns: they
-    // pay where a block has that many pixel-neighbours to look up.
-    const long long resident = (long long)FILTER_BLOCKS * sms, per_block = (long long)p.W * p.H * p.n / std::min(resident, work);
-    if (bytes <= FILTER_TABLE_BYTES && per_block >= 2ll * (long long)entries) {
+    // pay where a block has that many pixel-neighbours to look up (us a call, direct and
+    // tabulated: 1920x960 and 1 map, 1.4 look-ups an entry, 25.7 and 21.8; 960x480 and
+    // 1 map, 0.7, 7.8 and 7.5; 256x128 and 4 maps, 0.75, 4.7 and 4.9).
+    const long long per_block = (long long)p.W * p.H * p.n / blocks;
+    if (bytes <= FILTER_TABLE_BYTES && per_block >= (long long)entries) {
         if (bytes > 48 * 1024) {
             e = cudaFuncSetAttribute(filter_kernel<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, FILTER_TABLE_BYTES);
             if (e != cudaSuccess) return e;
         }
-        filter_kernel<true><<<(unsigned)std::min(resident, work), FILTER_THREADS, bytes, stream>>>(p, T);
+        filter_kernel<true><<<(unsigned)blocks, 32 * warps, bytes, stream>>>(p, T);
     } else {
-        filter_kernel<false><<<(unsigned)std::min<long long>(work, 1ll << 30), FILTER_THREADS, 0, stream>>>(p, T);
+        // (nothing to share: blocks of up to 4 warps, whose slots are free again sooner; 1920x960
+        // and 1 map 25.7 us, of 16 warps 26.9)
+        const int few = std::min(warps, 4);
+        filter_kernel<false><<<(unsigned)std::min<long long>((strips + few - 1) / few, 1ll << 30), 32 * few, 0, stream>>>(p, T);
     }
     return cudaGetLastError();
 }
