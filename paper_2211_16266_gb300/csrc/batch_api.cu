@@ -39,9 +39,7 @@ struct BatchEngine {
     std::map<TexKey, TexImage> tex;
     std::vector<DevBuffer> ref_stage, out_stage;
     DevBuffer d_problems, d_work, d_counters;
-    DevBuffer d_changed;         // change flags of every keyframe of the batch
-    bool exec_recorded = false;  // a stream being recorded took a replay: its d_changed is kept
-    std::vector<void*> retired;  // outgrown flags that such a recording holds
+    DevBuffer d_changed;  // change flags of every keyframe of the batch
     void* h_problems = nullptr;  // pinned copies read by the captured graph
     void* h_work = nullptr;
     size_t h_problems_bytes = 0, h_work_bytes = 0;
@@ -106,7 +104,6 @@ void batch_shutdown(pmsp_ctx* c) {
             if (d.ptr) cudaFree(d.ptr);
     for (DevBuffer* d : {&b.d_problems, &b.d_work, &b.d_counters, &b.d_changed})
         if (d->ptr) cudaFree(d->ptr);
-    for (void* p : b.retired) cudaFree(p);
     if (b.h_problems) cudaFreeHost(b.h_problems);
     if (b.h_work) cudaFreeHost(b.h_work);
     if (b.capture) cudaStreamDestroy(b.capture);
@@ -148,16 +145,14 @@ static std::vector<uint8_t> batch_signature(const pmsp_batch_item* items, int n,
 // Change flags of the batch's keyframes, n bytes in all, or NULL where there are
 // none (out of memory; a caller's recording, whose replays may overlap a later
 // batch): the half-sweeps then try every neighbour. `own`: the engine's capture,
-// which reuses the flags of the eager run before it.
+// which reuses the flags of the eager run before it. Its graph is replayed on the
+// context's stream only, and dropped before an eager batch moves the flags.
 static uint8_t* batch_flags(pmsp_ctx* c, BatchEngine& b, size_t n, cudaStream_t st, bool own) {
     DevBuffer& f = b.d_changed;
     if (own) return f.bytes >= n ? static_cast<uint8_t*>(f.ptr) : nullptr;
     if (recording(st)) return nullptr;
     if (f.bytes < n) {
-        if (f.ptr && b.exec_recorded) {
-            b.retired.push_back(f.ptr);
-            b.exec_recorded = false;
-        } else if (f.ptr) {
+        if (f.ptr) {
             cudaStreamSynchronize(c->stream);
             cudaFree(f.ptr);
         }
@@ -442,16 +437,14 @@ int pmsp_densify_batch(pmsp_ctx* c, const pmsp_batch_item* items, int n, uint32_
     if (graph) {
         std::vector<uint8_t> sig = batch_signature(items, n, t);
         if (b.exec && sig == b.signature) {
+            // A recorded replay would take the engine's change flags and plan along, which a
+            // later batch writes. The runtime refuses to record one; so does this call, and
+            // leaves the recording whole.
+            if (recording(c->stream)) return cuda_fail(c, cudaErrorStreamCaptureUnsupported, "graph launch");
             cudaError_t e = cudaGraphLaunch(b.exec, c->stream);
-            // the replay reads the pinned copies: mark it, unless the caller is recording
-            // the stream (an event recorded there could not be waited on afterwards)
-            cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
-            b.exec_recorded = b.exec_recorded || recording(c->stream);
-            if (e == cudaSuccess && cudaStreamIsCapturing(c->stream, &cap) == cudaSuccess &&
-                cap == cudaStreamCaptureStatusNone) {
-                if (!b.staged_ev) e = cudaEventCreateWithFlags(&b.staged_ev, cudaEventDisableTiming);
-                if (e == cudaSuccess) e = cudaEventRecord(b.staged_ev, c->stream);
-            }
+            // the replay reads the pinned copies: mark it
+            if (e == cudaSuccess && !b.staged_ev) e = cudaEventCreateWithFlags(&b.staged_ev, cudaEventDisableTiming);
+            if (e == cudaSuccess) e = cudaEventRecord(b.staged_ev, c->stream);
             return e == cudaSuccess ? PMSP_OK : cuda_fail(c, e, "graph launch");
         }
         drop_graph(b);
