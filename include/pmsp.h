@@ -295,8 +295,9 @@ int pmsp_view_filter(pmsp_ctx* ctx, const pmsp_pose* a, const pmsp_pose* b, cons
  *            cap = 0 to size the output)
  * Synchronous. Device memory, held by the context between calls: a hash table
  * of 16 bytes per slot (a power of two >= twice the input pixels up to 2^22,
- * then one >= a quarter of them; where the voxels do not fit, up to one >= twice
- * the pixels) and a bit per pixel. Errors: PMSP_EINVAL for NULL or mismatched
+ * then one >= a quarter of them), a bit per pixel and, once the voxels of a call
+ * did not fit, a second table (a power of two, one and a half to three slots per
+ * voxel that there could be). Errors: PMSP_EINVAL for NULL or mismatched
  * arguments, voxel <= 0, or a point beyond the key range.
  */
 int pmsp_fuse(pmsp_ctx* ctx, const pmsp_maps* maps, const pmsp_pose* poses, int n, float voxel, float* points,

@@ -19,7 +19,8 @@
 //   (16 bytes a slot, key and pixel in one sector; 6 keyframes at 1920x960 take
 //   64 MB, within L2, where two slots per pixel took 512 MB). The pixels left are
 //   listed per tile, so that full warps wait for the table together. A table that
-//   fills up is reported and the caller comes again with a larger one. 6 keyframes
+//   fills up is reported, with the candidates left, and the caller comes again with
+//   one that has room for them. 6 keyframes
 //   at 1920x960, 1 M voxels: 85 us insertion (was 198 over 6 launches), 33 us
 //   marks, scan and points (was 280), against 10 us for its 64 MB of maps, points
 //   and origins; the whole call with its count-only first pass 1.39 -> 0.45 ms.
@@ -81,7 +82,7 @@ __global__ void __launch_bounds__(FT_W * FT_H) fuse_insert_kernel(const __grid_c
     __shared__ float2 row[FT_H * FT_V], col[FT_W];  // (sin, cos) of latitude and longitude, as pixel_bearing
     __shared__ unsigned long long keys[FT_H * FT_V][FT_W];
     __shared__ unsigned short list[FT_H * FT_V * FT_W];
-    __shared__ unsigned claimed, full, listed;
+    __shared__ unsigned claimed, full, listed, missed;
     const int k = fuse_view(A, blockIdx.x), b = blockIdx.x - A.tile_base[k];
     const CloudView& V = A.views[k];
     const int tiles_x = (V.W + FT_W - 1) / FT_W;
@@ -103,9 +104,11 @@ __global__ void __launch_bounds__(FT_W * FT_H) fuse_insert_kernel(const __grid_c
             row[tid - FT_W] = make_float2(sn, cs);
         }
     } else if (tid == FT_W * FT_H - 1) {
-        claimed = listed = 0;
+        claimed = listed = missed = 0;
         full = *(volatile unsigned*)A.err & ERR_CAPACITY;  // the caller will come again: nothing more is worth doing
-        if (!full && *(volatile unsigned long long*)A.count > A.most_voxels) {
+        const unsigned long long now = *(volatile unsigned long long*)A.count, voxels = (unsigned)now, tiles = now >> 32;
+        if (!full && (voxels > A.most_voxels ||
+                      (A.foresee && 2 * tiles >= gridDim.x && 5 * voxels * gridDim.x > 6 * A.most_voxels * tiles))) {
             full = 1;
             atomicOr(A.err, ERR_CAPACITY);
         }
@@ -126,7 +129,6 @@ __global__ void __launch_bounds__(FT_W * FT_H) fuse_insert_kernel(const __grid_c
         keys[threadIdx.y + p * FT_H][threadIdx.x] = key[p];
     }
     __syncthreads();
-    if (full) return;
     // the tile's candidates in a list, so that the insertion runs with full warps
 #pragma unroll
     for (int p = 0; p < FT_V; ++p) {
@@ -141,6 +143,10 @@ __global__ void __launch_bounds__(FT_W * FT_H) fuse_insert_kernel(const __grid_c
         if (first) list[at] = (unsigned short)(y * FT_W + threadIdx.x);
     }
     __syncthreads();
+    if (full) {
+        if (tid == 0 && listed) atomicAdd(A.left, (unsigned long long)listed);
+        return;
+    }
     unsigned won = 0;
     for (int c = tid; c < (int)listed; c += FT_W * FT_H) {
         const int y = list[c] / FT_W, x = list[c] % FT_W;
@@ -159,17 +165,24 @@ __global__ void __launch_bounds__(FT_W * FT_H) fuse_insert_kernel(const __grid_c
             }
             s = (s + 1) & A.mask;
         }
-        if (probe == A.most_probes) atomicOr(A.err, ERR_CAPACITY);
+        if (probe == A.most_probes) {
+            atomicOr(A.err, ERR_CAPACITY);
+            atomicAdd(&missed, 1u);
+        }
     }
 #pragma unroll
     for (int o = 16; o > 0; o >>= 1) won += __shfl_xor_sync(0xffffffffu, won, o);
     if (threadIdx.x == 0 && won) atomicAdd(&claimed, won);
     __syncthreads();
-    if (tid == 0 && claimed) atomicAdd(A.count, (unsigned long long)claimed);
+    if (tid == 0) {
+        atomicAdd(A.count, (1ull << 32) | claimed);
+        if (missed) atomicAdd(A.left, (unsigned long long)missed);
+    }
 }
 
 // Sets the bit of every slot's pixel.
 __global__ void __launch_bounds__(256) fuse_mark_kernel(const __grid_constant__ FuseArgs A) {
+    if (*A.err & ERR_CAPACITY) return;  // the caller will come again
     for (unsigned long long s = (unsigned long long)blockIdx.x * 256 + threadIdx.x; s <= A.mask; s += (unsigned long long)gridDim.x * 256) {
         const ulonglong2 t = *reinterpret_cast<const ulonglong2*>(A.table + s);
         if (t.x == EMPTY) continue;
@@ -232,6 +245,7 @@ __global__ void __launch_bounds__(1024) fuse_scan_kernel(unsigned* sums, int gro
 // 133 -> 108, 1 of 1920x960 at 1.39M voxels 192 -> 181.
 __global__ void __launch_bounds__(SCAN_BLOCK) fuse_write_kernel(const __grid_constant__ FuseArgs A) {
     __shared__ unsigned ws[SCAN_BLOCK / 32], words[SCAN_BLOCK], before[SCAN_BLOCK];
+    if (*A.err & ERR_CAPACITY) return;
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     const int w0 = blockIdx.x * SCAN_BLOCK;
     const unsigned own = w0 + threadIdx.x < A.n_words ? A.bits[w0 + threadIdx.x] : 0;
@@ -341,7 +355,7 @@ int fuse_tiles(int W, int H) { return ((W + FT_W - 1) / FT_W) * ((H + FT_H * FT_
 
 cudaError_t launch_fuse(const FuseArgs& a, cudaStream_t stream) {
     cudaError_t e = cudaMemsetAsync(a.table, 0xff, (a.mask + 1) * sizeof(FuseSlot), stream);
-    if (e == cudaSuccess) e = cudaMemsetAsync(a.count, 0, 2 * sizeof(unsigned long long), stream);  // and the error word
+    if (e == cudaSuccess) e = cudaMemsetAsync(a.count, 0, 3 * sizeof(unsigned long long), stream);  // and the words after it
     if (e != cudaSuccess) return e;
     fuse_insert_kernel<<<a.tile_base[a.n], dim3(FT_W, FT_H), 0, stream>>>(a);
     if (a.cap > 0) {  // else the count is all that is asked for

@@ -102,11 +102,16 @@ int pmsp_fuse(pmsp_ctx* c, const pmsp_maps* maps, const pmsp_pose* poses, int n,
     }
     if (total >= (1ll << 31)) return ctx_fail(c, PMSP_EINVAL, "too many pixels to fuse in one call");
     // The table has two slots per pixel as long as that is 2^22 slots (64 MB, half
-    // the L2) or less; beyond, it starts there or at a slot for every fourth pixel
-    // (dense maps put several pixels into a voxel) and grows fourfold, to at most two
-    // per pixel, as long as the insertion reports it too small. Both calls (count, then
-    // points) over 1 keyframe of 1920x960 at 622,810 voxels take 245 us so, 657 from a
-    // slot for every fourth pixel on; 3 keyframes at 3.85M voxels, where it grows, 1255.
+    // the L2) or less; beyond, 2^22 or a slot for every fourth pixel (dense maps put
+    // several pixels into a voxel). Both calls (count, then points) over 1 keyframe of
+    // 1920x960 at 622,810 voxels take 245 us so, 657 from a slot for every fourth pixel on.
+    // Where the insertion finds the table too small, it comes again with one and a half
+    // slots for each voxel there can be, and up to 2^23 pixels, where a table of two slots
+    // per pixel costs little more, the attempt that fails ends early: from half of the tiles on
+    // the voxels so far tell, with a fifth to spare. 3 keyframes of 1920x960, one call: 3.70M
+    // voxels 515 us (an attempt to its end, then a table four times as large: 730; two
+    // slots per pixel at once, every pixel inserted: 605), 4.07M 555 (770, 622), 3.27M, where
+    // the attempt is not cut short, 567 (665, 590). 6 keyframes at 8.18M voxels 920 (990, 1340).
     constexpr unsigned long long IN_L2 = 1ull << 22;
     unsigned long long slots = 1024, most = 1024;
     while (most < 2ull * (unsigned long long)total) most <<= 1;
@@ -115,80 +120,91 @@ int pmsp_fuse(pmsp_ctx* c, const pmsp_maps* maps, const pmsp_pose* poses, int n,
     const bool host = memory == PMSP_HOST;
     const long long kept_max = cap < total ? cap : total;
     const int n_words = (int)((total + 31) / 32);
+    // context buffers: hash table | bits | block sums | count, error, left | host staging
+    const size_t t_bytes = rounded(slots * sizeof(FuseSlot)), b_bytes = rounded((size_t)n_words * sizeof(unsigned));
+    const size_t s_bytes = rounded(((size_t)n_words / 256 + 1) * sizeof(unsigned));
+    const size_t c_bytes = rounded(3 * sizeof(unsigned long long));
+    size_t h_bytes = 0;
+    if (host)
+        h_bytes = rounded((size_t)total * sizeof(float)) + rounded((size_t)kept_max * 3 * sizeof(float)) +
+                  rounded((size_t)kept_max * sizeof(long long));
+    int rc;
+    if ((rc = ensure_buffer(c, c->cloud_table, t_bytes + b_bytes + s_bytes + c_bytes + h_bytes))) return rc;
+    char* base = static_cast<char*>(c->cloud_table.ptr);
     FuseArgs A;
     memset(&A, 0, sizeof A);
-    unsigned long long res[2] = {0, 0};
-    int rc;
-    for (;;) {
-        // context buffers: hash table | bits | block sums | count + error | host staging
-        const size_t t_bytes = rounded(slots * sizeof(FuseSlot)), b_bytes = rounded((size_t)n_words * sizeof(unsigned));
-        const size_t s_bytes = rounded(((size_t)n_words / 256 + 1) * sizeof(unsigned));
-        const size_t c_bytes = rounded(2 * sizeof(unsigned long long));
-        size_t h_bytes = 0;
-        if (host)
-            h_bytes = rounded((size_t)total * sizeof(float)) + rounded((size_t)kept_max * 3 * sizeof(float)) +
-                      rounded((size_t)kept_max * sizeof(long long));
-        if ((rc = ensure_buffer(c, c->cloud_table, t_bytes + b_bytes + s_bytes + c_bytes + h_bytes))) return rc;
-        char* base = static_cast<char*>(c->cloud_table.ptr);
-        A.table = reinterpret_cast<FuseSlot*>(base);
-        A.mask = slots - 1;
-        A.most_probes = slots < most ? 128 : slots;
-        A.most_voxels = slots < most ? slots - slots / 4 : slots;
-        A.bits = reinterpret_cast<unsigned*>(base + t_bytes);
-        A.n_words = n_words;
-        A.sums = reinterpret_cast<unsigned*>(base + t_bytes + b_bytes);
-        A.count = reinterpret_cast<unsigned long long*>(base + t_bytes + b_bytes + s_bytes);
-        A.err = reinterpret_cast<unsigned*>(A.count + 1);
-        char* hs = base + t_bytes + b_bytes + s_bytes + c_bytes;
-        A.inv_voxel = 1.0f / voxel;
-        A.cap = cap;
-        A.points = points;
-        A.src = reinterpret_cast<long long*>(src);
+    A.bits = reinterpret_cast<unsigned*>(base + t_bytes);
+    A.n_words = n_words;
+    A.sums = reinterpret_cast<unsigned*>(base + t_bytes + b_bytes);
+    A.count = reinterpret_cast<unsigned long long*>(base + t_bytes + b_bytes + s_bytes);
+    A.err = reinterpret_cast<unsigned*>(A.count + 1);
+    A.left = A.count + 2;
+    char* hs = base + t_bytes + b_bytes + s_bytes + c_bytes;
+    A.inv_voxel = 1.0f / voxel;
+    A.cap = cap;
+    A.points = points;
+    A.src = reinterpret_cast<long long*>(src);
+    if (host) {
+        A.points = reinterpret_cast<float*>(hs + rounded((size_t)total * sizeof(float)));
+        A.src = src ? reinterpret_cast<long long*>(hs + rounded((size_t)total * sizeof(float)) +
+                                                   rounded((size_t)kept_max * 3 * sizeof(float)))
+                    : nullptr;
+        A.cap = kept_max;
+    }
+    A.n = n;
+    long long off = 0;
+    int tiles = 0;
+    for (int k = 0; k < n; ++k) {
+        CloudView& V = A.views[k];
+        V.W = maps[k].w;
+        V.H = maps[k].h;
+        V.depth = maps[k].depth;
+        const size_t px = (size_t)V.W * V.H;
         if (host) {
-            A.points = reinterpret_cast<float*>(hs + rounded((size_t)total * sizeof(float)));
-            A.src = src ? reinterpret_cast<long long*>(hs + rounded((size_t)total * sizeof(float)) +
-                                                       rounded((size_t)kept_max * 3 * sizeof(float)))
-                        : nullptr;
-            A.cap = kept_max;
+            float* d = reinterpret_cast<float*>(hs) + off;
+            if ((rc = stage_in(c, maps[k].depth, px, d))) return rc;
+            V.depth = d;
         }
-        A.n = n;
-        long long off = 0;
-        int tiles = 0;
-        for (int k = 0; k < n; ++k) {
-            CloudView& V = A.views[k];
-            V.W = maps[k].w;
-            V.H = maps[k].h;
-            V.depth = maps[k].depth;
-            const size_t px = (size_t)V.W * V.H;
-            if (host) {  // (a larger buffer moved the staging)
-                float* d = reinterpret_cast<float*>(hs) + off;
-                if ((rc = stage_in(c, maps[k].depth, px, d))) return rc;
-                V.depth = d;
-            }
-            for (int j = 0; j < 9; ++j) V.R[j] = (float)poses[k].R[j];
-            for (int j = 0; j < 3; ++j) V.t[j] = (float)poses[k].t[j];
-            A.base[k] = off;
-            A.tile_base[k] = tiles;
-            off += (long long)px;
-            tiles += fuse_tiles(V.W, V.H);
-        }
-        A.base[n] = off;
-        A.tile_base[n] = tiles;
+        for (int j = 0; j < 9; ++j) V.R[j] = (float)poses[k].R[j];
+        for (int j = 0; j < 3; ++j) V.t[j] = (float)poses[k].t[j];
+        A.base[k] = off;
+        A.tile_base[k] = tiles;
+        off += (long long)px;
+        tiles += fuse_tiles(V.W, V.H);
+    }
+    A.base[n] = off;
+    A.tile_base[n] = tiles;
+    auto insert = [&](FuseSlot* table, unsigned long long size, unsigned long long (&res)[3]) {
+        A.table = table;
+        A.mask = size - 1;
         cudaError_t e = launch_fuse(A, c->stream);
         if (e != cudaSuccess) return cuda_fail(c, e, "fuse launch");
         e = cudaMemcpyAsync(res, A.count, sizeof res, cudaMemcpyDeviceToHost, c->stream);
         if (e == cudaSuccess) e = cudaStreamSynchronize(c->stream);
-        if (e != cudaSuccess) return cuda_fail(c, e, "fuse read-back");
-        if (((unsigned)res[1] & ERR_RANGE) || !((unsigned)res[1] & ERR_CAPACITY) || slots >= most) break;
-        slots = std::min(most, slots * 4);
+        return e == cudaSuccess ? (int)PMSP_OK : cuda_fail(c, e, "fuse read-back");
+    };
+    const bool fits = slots >= most;
+    A.most_probes = fits ? slots : 128;
+    A.most_voxels = fits ? slots : slots - slots / 4;
+    A.foresee = !fits && total <= (1ll << 23);
+    unsigned long long res[3] = {0, 0, 0};
+    if ((rc = insert(reinterpret_cast<FuseSlot*>(base), slots, res))) return rc;
+    if (((unsigned)res[1] & ERR_CAPACITY) && !((unsigned)res[1] & ERR_RANGE) && !fits) {
+        const unsigned long long voxels = (unsigned)res[0] + res[2];  // at most
+        while (2 * slots < 3 * voxels) slots <<= 1;
+        if ((rc = ensure_buffer(c, c->cloud_large, slots * sizeof(FuseSlot)))) return rc;
+        A.most_probes = A.most_voxels = slots;
+        A.foresee = false;
+        if ((rc = insert(static_cast<FuseSlot*>(c->cloud_large.ptr), slots, res))) return rc;
     }
     cudaError_t e = cudaSuccess;
     const unsigned err = (unsigned)res[1];
     if (err & ERR_RANGE) return ctx_fail(c, PMSP_EINVAL, "a point lies more than 2^20 voxels from the origin");
     if (err) return ctx_fail(c, PMSP_EDEVICE, "fuse error flag 0x%x", err);
-    *count = (int64_t)res[0];
+    const long long voxels = (long long)(unsigned)res[0];
+    *count = voxels;
     if (host) {
-        const long long kept = (long long)res[0] < kept_max ? (long long)res[0] : kept_max;
+        const long long kept = voxels < kept_max ? voxels : kept_max;
         if (kept > 0) {
             e = cudaMemcpyAsync(points, A.points, (size_t)kept * 3 * sizeof(float), cudaMemcpyDeviceToHost, c->stream);
             if (e == cudaSuccess && src)

@@ -140,14 +140,16 @@ struct FuseArgs {
     FuseSlot* table;
     unsigned long long mask;         // table capacity - 1 (capacity a power of two)
     unsigned long long most_probes, most_voxels;  // beyond either the table counts as too small
+    bool foresee;                    // whether it will be too small is judged from half of the tiles on
     unsigned* bits;                  // a bit per pixel: kept
     int n_words;
     unsigned* sums;                  // kept pixels per group of 256 words, then before it
     float* points;                   // output: 3 floats per kept point
     long long* src;                  // output (optional): keyframe << 32 | pixel
     long long cap;                   // output capacity in points
-    unsigned long long* count;       // voxels; the error word follows it
+    unsigned long long* count;       // tiles done << 32 | voxels; the next two words follow it
     unsigned* err;
+    unsigned long long* left;        // candidates that a table too small left out
 };
 
 struct CompletenessArgs {

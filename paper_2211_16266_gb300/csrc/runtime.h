@@ -73,7 +73,8 @@ struct pmsp_ctx {
     std::vector<pmsp::TexImage> src_tex;  // one texture per source slot
     pmsp::TexImage sample_tex;
     pmsp::DevBuffer ref_stage, map_stage, filter_stage, sample_stage, median_stage;
-    pmsp::DevBuffer cloud_table, cloud_stage;  // fusion (hash table, marks, staging); view filter, completeness
+    pmsp::DevBuffer cloud_table, cloud_large;  // fusion: hash table, marks, staging; the table of calls that it was too small for
+    pmsp::DevBuffer cloud_stage;               // view filter, completeness
     pmsp::DevBuffer changed;                   // change flags of the running densification
     pmsp::DevBuffer warp_zbuf, warp_prev;  // plane-map warping: claims, staged previous maps
     pmsp::Serving* serving = nullptr;

@@ -67,7 +67,7 @@ def test_tile_edges_and_small_inputs(pm, sizes, voxel):
 
 
 # few enough pixels that a table seen to be too small is left early, and too many for that
-@pytest.mark.parametrize("sizes", [[(2048, 1024), (2050, 1025)], [(2048, 1024), (2050, 1025), (2047, 1023)]])
+@pytest.mark.parametrize("sizes", [[(2048, 1024), (2040, 1024)], [(2048, 1024), (2050, 1025), (2047, 1023)]])
 @pytest.mark.parametrize("host", [False, True])
 def test_a_table_too_small(pm, sizes, host):
     depths, poses = _views(sizes, 5)
