@@ -168,6 +168,11 @@ void pmsp_default_params(pmsp_params* p);
  *   out                  w x h of the reference; depth, normal, cost all required.
  * Returns PMSP_EINVAL for an odd width or height, best_k outside [1, n_src], a
  * bad window, a bad range, a NULL pointer or an unknown format.
+ * Device memory, held by the context between calls: a texture array per source
+ * and, for what a run remembers of its half-sweeps, a byte per reference pixel and
+ * two 4-byte words per iteration (pmsp_densify_warped shares it). Where that memory
+ * cannot be had, and in a call that the caller records into a graph, the run goes
+ * without: the same maps, with every neighbour tried in every half-sweep.
  */
 int pmsp_densify(pmsp_ctx* ctx, const pmsp_image* ref, const pmsp_pose* ref_pose,
                  const pmsp_image* srcs, const pmsp_pose* src_poses, int n_src,
@@ -420,6 +425,11 @@ typedef struct {
  * the context reuses: a call made while the previous call's upload (or graph
  * replay) is still queued waits on the host until that has run. The first
  * capture of a PMSP_BATCH_GRAPH batch waits for the context stream to idle.
+ * While the caller records the context's stream, a PMSP_BATCH_GRAPH batch is
+ * refused (PMSP_ECUDA); one without the flag is recorded launch by launch.
+ * Device memory, held by the context between calls: a texture array per source
+ * buffer and, summed over the batch, what pmsp_densify remembers of a run (none in
+ * a recorded batch).
  */
 int pmsp_densify_batch(pmsp_ctx* ctx, const pmsp_batch_item* items, int n, uint32_t flags,
                        const pmsp_tuning* tuning);

@@ -1036,13 +1036,17 @@ __device__ __forceinline__ void sweep_pooled(const PixelParams& P, SM& sm, int b
 // A refinement candidate's cost must fall below the incumbent's to matter, and
 // most end far above it. After part of the samples the cost is already bounded
 // from below: over the samples A taken so far let V_I, V_J and C be the weighted
-// variances and covariance; whatever the source shows at the others, the best it
-// can do is follow the reference exactly, J = a + b I, so with the residual
-// r = (V_I - C^2 / V_J) / Sw_A of the samples taken (V_I / Sw_A where C <= 0,
-// scaled sums as below) and the whole window's V = varI / Sw,
-//   NCC^2 <= V / (V + r),
+// variances and covariance. (1 - NCC^2) V is what the best line in J leaves of the
+// reference's sum of squares V = varI / Sw over the whole window, and over A alone
+// a line of positive slope leaves at least r = (V_I - C^2 / V_J) / Sw_A (V_I / Sw_A where
+// C <= 0, scaled sums as below). So for NCC > 0
+//   NCC^2 <= 1 - r / V <= V / (V + r),
 // and the cost is at least the mean of 1 - NCC over the best_k views of highest
-// bound. A candidate whose bound clears the incumbent is dropped; the others
+// bound. The last form is the one used. Its root has the smaller rounding error (a
+// derivative of at most 1/2 in r / V, where that of 1 - r / V grows without limit), but
+// it is not the sharpest: r <= V, so a view's bound never exceeds 1 - sqrt(1/2) = 0.293,
+// and an incumbent above that lets no test go.
+// A candidate whose bound clears the incumbent is dropped; the others
 // are evaluated to the end by the same operations in the same order as ever, so
 // the maps do not change.
 //
@@ -1150,8 +1154,9 @@ __device__ __forceinline__ bool neighbour_from_tables(const PixelParams& P, cons
 // after 2.5 of 6 rows on average; lanes left idle and the hand-out keep a third of
 // that from the clock. 1920x960, 6 views, 8 iterations: 75.9 -> 66.8 ms; 4 views at
 // 960x480 14.7 -> 13.5 ms; 3840x1920, 8 views without noise, 4 iterations 229 ->
-// 206 ms. With sensor noise (costs around 0.4) the bound drops nothing and the hand-
-// out costs 6 %, so such half-sweeps stay with the pooled kernel (bounded_turn).
+// 206 ms. Where costs stay above what the bound can reach (0.293, refine_margin; around 0.4
+// with sensor noise at 3840x1920) it drops nothing and the hand-out costs 6 %, so
+// such half-sweeps stay with the pooled kernel (bounded_turn).
 template <int NS, class VA, int WIN, class SM>
 __device__ __forceinline__ void sweep_bounded(const PixelParams& P, SM& sm, int bx, int by, int colour, int iter) {
     constexpr int NP = NS / 2, NPA = NP > 0 ? NP : 1;
