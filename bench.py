@@ -244,7 +244,8 @@ def run_gpu(args):
         config=keyframe_config(ws),
         latency_ms=dict(p50=float(np.percentile(times, 50)), p99=float(np.percentile(times, 99))),
         hypothesis_evals_per_s=ws * evals * args.steps / (total_ms / 1e3),
-        gpu_launches=args.steps * (2 + 2 * ITERS + 1),
+        # initialisation, every half-sweep's pooled kernel, the bounded one beside all but the first, the filter
+        gpu_launches=args.steps * (1 + 2 * ITERS + (2 * ITERS - 1) + 1),
         clocks=clocks,
     )
     if rank == 0:
