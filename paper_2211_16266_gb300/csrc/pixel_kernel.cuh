@@ -1149,8 +1149,9 @@ __device__ __forceinline__ bool neighbour_from_tables(const PixelParams& P, cons
 // order; a success makes the tests started from the older incumbent void, and
 // they are started again.
 //
-// Bound, like sweep_pooled, by FP32 issue of the samples taken (367 instructions a
-// sample of 6 views). On a converged 960x480 keyframe of 6 views a test is dropped
+// Bound, like sweep_pooled, by FP32 issue of the samples taken (1920x960, 6 views: 415
+// warp instructions a sample with the bound and the hand-out, 25 of 32 lanes active;
+// sweep_pooled 346 and 31.4). On a converged 960x480 keyframe of 6 views a test is dropped
 // after 2.5 of 6 rows on average; lanes left idle and the hand-out keep a third of
 // that from the clock. 1920x960, 6 views, 8 iterations: 75.9 -> 66.8 ms; 4 views at
 // 960x480 14.7 -> 13.5 ms; 3840x1920, 8 views without noise, 4 iterations 229 ->
