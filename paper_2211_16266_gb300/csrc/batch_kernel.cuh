@@ -63,10 +63,16 @@ __global__ void __launch_bounds__(BLOCK_THREADS, min_blocks_for(MAXS)) batch_ker
     }
 }
 
+// Instances whose shared-memory split is set (prefer_texture_cache): the one above 10 views,
+// which gathers view by view. 3 keyframes of 960x480, 4 iterations, ms with the split
+// set and left to the driver: 12 views 146.8 and 150.4, 10 views 62.05 and 61.98, 6 views 38.37
+// both, 4 views 28.57 and 27.76, 2 views 16.58 and 16.53.
+constexpr bool batch_prefers_texture_cache(int maxs) { return maxs > 10; }
+
 template <int MAXS>
 int batch_kernel_blocks_per_sm_t() {
     int n = 0;
-    prefer_texture_cache<batch_kernel<MAXS>>();
+    if (batch_prefers_texture_cache(MAXS)) prefer_texture_cache<batch_kernel<MAXS>>();
     if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, batch_kernel<MAXS>, BLOCK_THREADS, 0) != cudaSuccess)
         return 1;
     return n > 0 ? n : 1;
@@ -75,7 +81,7 @@ int batch_kernel_blocks_per_sm_t() {
 template <int MAXS>
 cudaError_t launch_batch_kernel_t(const BatchArgs& a, int grid, cudaStream_t stream) {
     if (a.n_work <= 0) return cudaSuccess;
-    prefer_texture_cache<batch_kernel<MAXS>>();
+    if (batch_prefers_texture_cache(MAXS)) prefer_texture_cache<batch_kernel<MAXS>>();
     batch_kernel<MAXS><<<grid, BLOCK_THREADS, 0, stream>>>(a);
     return cudaGetLastError();
 }
